@@ -376,10 +376,12 @@ int bspai_gmres(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_t u_g, b
  * memory), 1 = k_mgs_res (the new vector held on chip; per_thread rows per
  * thread), 2 = k_mgs_res2 (fp32, the new vector in registers; per_thread
  * pairs of adjacent rows per thread); block_threads and blocks give the
- * launch; poll_bulk = 1 when the on-chip kernel's warp 0 reads the grid
- * reductions' slots by bulk copies into shared memory instead of by loads
- * (at least 16 KB of each basis vector per block and at least 64 blocks),
- * 0 otherwise.  A query only: nothing is launched or allocated.  n < 1:
+ * launch (the blocks that hold rows; where an SM is free, one more block
+ * applies the Givens rotations); poll_bulk = 1 when the on-chip kernel reads
+ * the grid reductions' slots by bulk copies into shared memory instead of by
+ * loads (at least 16 KB of each basis vector per block and at least 64
+ * blocks), 0 otherwise.  Every kernel takes the basis in groups of 1 to 8
+ * vectors, one reduction per group.  A query only: nothing is launched or allocated.  n < 1:
  * BSPAI_ERR_INVALID; another u_g: BSPAI_ERR_UNSUPPORTED. */
 typedef struct {
     int32_t kernel;
@@ -406,7 +408,7 @@ int bspai_gmres_b(bspai_A_h A, bspai_BM_h A_bucketed, bspai_BM_h BM, const doubl
  * changes where the workspace lives.
  *   - Workspace: one fixed 64 MiB block of device memory that belongs to the
  *     library image (every GPU that loads the library holds it until the
- *     process exits).  The call needs n_pad * (kmax + 1) values in u_g
+ *     process exits; 1 MiB beside it holds the reductions' slots).  The call needs n_pad * (kmax + 1) values in u_g
  *     (n_pad = n rounded up to 64) plus about 8 (kmax + 1)^2 bytes; larger
  *     problems are rejected with BSPAI_ERR_INVALID and a message giving the
  *     bytes needed, and nothing is launched.

@@ -10,59 +10,23 @@
 // only reads the flag between chunks.  Steps enqueued after convergence
 // return immediately.
 //
-// k_mgs keeps one contiguous range of rows per block.  Modified Gram-Schmidt
-// needs the j+1 dot products in sequence; pass i fuses the update by the
-// previous coefficient with the next dot product, z <- z - h_{i-1} v_{i-1};
-// partial += v_i . z, so each basis vector is streamed once per step.  The
-// block partial sums go to a global array, one grid barrier, and every block
-// then adds the partials in the same fixed order, so all blocks hold the same
-// h_ij (deterministic, no atomics).  The last pass forms ||z||_2 and
-// normalises v_{j+1}; block 0 then applies the Givens rotations (fp64) and
-// tests |g_{j+1}| <= tau ||M r||_2.  j + 2 barriers per step, each bounded in
-// time (BSPAI_TIMEOUT).
+// The MGS kernels keep one contiguous range of rows per block and take the basis
+// in groups of a few vectors, one grid-wide reduction per group (mgs.cuh): the
+// partial sums v_t . z of a group's vectors, then z -= sum h_t v_t.  Every block
+// adds the partials in the same fixed order, so all blocks hold the same h_ij
+// (deterministic, no atomics).  The last pass forms ||z||_2 and normalises
+// v_{j+1}; the Givens rotations (fp64) and the test |g_{j+1}| <= tau ||M r||_2
+// follow.  Every wait is bounded in time (BSPAI_TIMEOUT).
 #include <cmath>
 #include <cstring>
 #include <mutex>
 #include <vector>
 
 #include "common.cuh"
+#include "mgs.cuh"
 #include "tags.cuh"
 
 namespace bspai {
-
-struct GmresState {
-    int j;        // completed Arnoldi steps (= k)
-    int done;     // 1 once converged, broken down, failed or at kmax
-    int status;   // BSPAI_OK, BSPAI_TIMEOUT, BSPAI_NONFINITE
-    int kmax;
-    double beta;  // ||M r||_2 (in u_g)
-    double tau;
-    double target;  // > 0: stop at |g| <= target instead of the tau test (restarted cycles)
-    double res;   // |g_k|
-    double hlast;
-    GridBar bar;
-};
-
-template <typename T>
-struct Ar;
-template <>
-struct Ar<float> {
-    static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-    static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-    static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-    static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
-    static __device__ __forceinline__ float sqrt(float a) { return __fsqrt_rn(a); }
-    static __device__ __forceinline__ float from(double a) { return __double2float_rn(a); }
-};
-template <>
-struct Ar<double> {
-    static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
-    static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
-    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
-    static __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
-    static __device__ __forceinline__ double sqrt(double a) { return __dsqrt_rn(a); }
-    static __device__ __forceinline__ double from(double a) { return a; }
-};
 
 __global__ void k_state_init(GmresState* st, int kmax, double tau, double target) {
     st->j = 0;
@@ -145,112 +109,132 @@ __global__ void __launch_bounds__(512) k_gmres_start(T* __restrict__ V, int n, G
     }
 }
 
-// The new rotation of step j from the swept column (hc[j] = carry, the entry the
-// earlier rotations handed on, hc[j+1] = hn = h_{j+1,j}), the update of g and
-// the tau test (fp64)
-__device__ void givens_finish(int j, int kmax, double hn, double carry, double* __restrict__ hc, double* cs,
-                              double* sn, double* g, GmresState* st) {
-    hc[j] = carry;
-    hc[j + 1] = hn;
-    const double a = carry, b = hn;
-    const double rr = __dsqrt_rn(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b)));
-    double c = 1.0, s = 0.0;
-    if (rr != 0.0) {
-        c = __ddiv_rn(a, rr);
-        s = __ddiv_rn(b, rr);
-    }
-    cs[j] = c;
-    sn[j] = s;
-    hc[j] = rr;
-    hc[j + 1] = 0.0;
-    g[j + 1] = __dmul_rn(-s, g[j]);
-    g[j] = __dmul_rn(c, g[j]);
-    const double res = fabs(g[j + 1]);
-    const int k = j + 1;
-    const bool fin = isfinite(res) && isfinite(hn) && isfinite(rr);
-    st->res = res;
-    st->hlast = hn;
-    st->j = k;
-    if (!fin) st->status = BSPAI_NONFINITE;
-    const double lvl = st->target > 0.0 ? st->target : __dmul_rn(st->tau, st->beta);
-    st->done = (res <= lvl) || hn == 0.0 || k >= kmax || !fin;
-}
-
-// rotation i of the earlier steps applied to the pair (carry, h_{i+1,j}): the
-// rotated h_{i,j} is returned, the entry handed on to rotation i + 1 stays in carry
-__device__ __forceinline__ double givens_apply(double ci, double si, double& carry, double hi1) {
-    const double t1 = __dadd_rn(__dmul_rn(ci, carry), __dmul_rn(si, hi1));
-    carry = __dadd_rn(__dmul_rn(-si, carry), __dmul_rn(ci, hi1));
-    return t1;
-}
-
-// Givens rotations on column j of H (written unrotated), update of g and the tau test (fp64)
-__device__ void givens_step(int j, int kmax, double hn, double* H, double* cs, double* sn, double* g,
-                            GmresState* st) {
-    double* __restrict__ hc = H + (int64_t)j * (kmax + 1);
-    const double* __restrict__ c_ = cs;
-    const double* __restrict__ s_ = sn;
-    // the previous rotations applied to the new column; the entry each rotation hands
-    // to the next stays in a register, so only the running value is a dependent chain
-    // (the stored coefficients and column entries are independent loads)
-    double carry = hc[0];
-    for (int i = 0; i < j; ++i) hc[i] = givens_apply(c_[i], s_[i], carry, hc[i + 1]);
-    givens_finish(j, kmax, hn, carry, hc, cs, sn, g, st);
-}
-
+// MGS step of the orders whose rows do not fit on chip: the group's vectors and z
+// are streamed from memory.  Pass g takes the previous group out of z and forms
+// the products with the next group in one sweep, so a group of four costs ten
+// vector streams (four of each group, z read and written) where one vector at a
+// time costs sixteen.
+// (fp64 keeps one block per SM: the grid, which k_gmres_start shares, fixes the
+// order in which ||M r||_2 is summed.)
+constexpr int kStreamGB = 4;
 template <typename T>
-__global__ void __launch_bounds__(512) k_mgs(T* __restrict__ V, int64_t ldv, int n, GmresState* st, double* H,
-                                             double* cs, double* sn, double* g, T* part, unsigned long long tmo) {
+__global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_mgs(T* __restrict__ V, int64_t ldv, int n, GmresState* st, double* H,
+                                             double* cs, double* sn, double* g, T* part, T* tri,
+                                             unsigned long long* hq, unsigned long long tmo) {
+    constexpr int GB = kStreamGB;
     __shared__ int s_j, s_done, s_kmax;
+    __shared__ unsigned s_seq;
+    __shared__ T s_w[2 * GB][32], s_tot[2 * GB], s_h[GB], s_tri[GB][GB];
     if (threadIdx.x == 0) {
         s_j = st->j;
         s_done = st->done;
         s_kmax = st->kmax;
+        s_seq = *(volatile unsigned*)&st->bar.seq;
     }
     __syncthreads();
     if (s_done) return;
     const int j = s_j, kmax = s_kmax;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned tag = s_seq + 1u;
     int64_t r0, r1;
     block_rows(n, r0, r1);
     T* z = V + (int64_t)(j + 1) * ldv;
-    T hprev = T(0);
-    for (int i = 0; i <= j + 1; ++i) {
-        const T* vi = V + (int64_t)(i <= j ? i : j) * ldv;
-        const T* vp = V + (int64_t)(i > 0 ? i - 1 : 0) * ldv;
-        T acc = T(0);
-        if (i == 0) {
-            for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x)
-                acc = Ar<T>::add(acc, Ar<T>::mul(vi[r], z[r]));
-        } else if (i <= j) {
-            for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-                const T zr = Ar<T>::sub(z[r], Ar<T>::mul(hprev, vp[r]));
-                z[r] = zr;
-                acc = Ar<T>::add(acc, Ar<T>::mul(vi[r], zr));
+    const int ng = j / GB + 1;
+    T hp[GB];
+#pragma unroll
+    for (int t = 0; t < GB; ++t) hp[t] = T(0);
+    for (int gi = 0; gi <= ng; ++gi) {  // pass ng: the last group out of z, ||z||^2
+        const int i0 = gi * GB;
+        const bool last = gi == ng - 1, norm = gi == ng;
+        const int cnt = norm ? 0 : last ? j - i0 + 1 : GB;
+        const int have = gi > 0 ? (norm ? j + 1 - (i0 - GB) : GB) : 0;  // vectors of the previous group
+        T a[GB], q[GB], zz = T(0);
+#pragma unroll
+        for (int t = 0; t < GB; ++t) a[t] = q[t] = T(0);
+        for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
+            T v[GB], pv[GB];
+            T zr = z[r];
+#pragma unroll
+            for (int t = 0; t < GB; ++t) {
+                pv[t] = t < have ? V[(int64_t)(i0 - GB + t) * ldv + r] : T(0);
+                v[t] = t < cnt ? V[(int64_t)(i0 + t) * ldv + r] : T(0);
             }
-        } else {
-            for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-                const T zr = Ar<T>::sub(z[r], Ar<T>::mul(hprev, vp[r]));
+            if (have) {
+#pragma unroll
+                for (int t = 0; t < GB; ++t) zr = pk_nfma(hp[t], pv[t], zr);
                 z[r] = zr;
-                acc = Ar<T>::add(acc, Ar<T>::mul(zr, zr));
+            }
+            if (norm) {
+                zz = Ar<T>::fma(zr, zr, zz);
+            } else {
+                T vj = v[0];
+#pragma unroll
+                for (int t = 1; t < GB; ++t)
+                    if (t == cnt - 1) vj = v[t];
+#pragma unroll
+                for (int t = 0; t < GB; ++t) {
+                    a[t] = Ar<T>::fma(v[t], zr, a[t]);
+                    if (last) q[t] = Ar<T>::fma(v[t], vj, q[t]);
+                }
             }
         }
-        bool ok;
-        const T h = grid_sum(acc, part, i & 1, &st->bar, tmo, ok);
-        if (!ok) {
+        if (norm) a[0] = zz;
+        warp_multi_sum<GB>(a);
+        warp_multi_sum<GB>(q);
+        if ((lane & (32 / GB - 1)) == 0) {
+            s_w[warp_multi_index<GB>(lane)][w] = a[0];
+            s_w[GB + warp_multi_index<GB>(lane)][w] = q[0];
+        }
+        __syncthreads();
+        if (w < 2 * GB) {
+            T t = lane < (int)(blockDim.x >> 5) ? s_w[w][lane] : T(0);
+            t = warp_sum(t);
+            if (lane == 0) part[((int64_t)(gi & 1) * 2 * GB + w) * gridDim.x + blockIdx.x] = t;
+        }
+        if (!grid_sync(&st->bar, tmo)) {
             if (blockIdx.x == 0 && threadIdx.x == 0) {
                 st->status = BSPAI_TIMEOUT;
                 st->done = 1;
             }
             return;
         }
-        if (i <= j) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) H[(int64_t)j * (kmax + 1) + i] = (double)h;
-            hprev = h;
-        } else {
-            const T hn = Ar<T>::sqrt(h);
-            if (hn > T(0) && isfinite((double)hn))
-                for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) z[r] = Ar<T>::div(z[r], hn);
-            if (blockIdx.x == 0 && threadIdx.x == 0) givens_step(j, kmax, (double)hn, H, cs, sn, g, st);
+        if (w < 2 * GB) {
+            T t = T(0);
+            for (int b = lane; b < (int)gridDim.x; b += 32)
+                t = Ar<T>::add(t, *(volatile T*)&part[((int64_t)(gi & 1) * 2 * GB + w) * gridDim.x + b]);
+            t = warp_sum(t);
+            if (lane == 0) s_tot[w] = t;
+        }
+        __syncthreads();
+        if (norm) break;
+        if (w == 0) {
+            T row[GB];
+            group_rows<T, GB>(row, tri + (int64_t)i0 * GB, last ? cnt - 1 : cnt);
+            const T h = group_coeff<T, GB>(row, s_tot, cnt, last);
+            if (lane < GB) s_h[lane] = lane < cnt ? h : T(0);
+            if (blockIdx.x == 0) {
+                if (lane < cnt) tag_publish(h, hq + (int64_t)(i0 + lane) * TagWords<T>::W, tag);
+                if (last) group_new_row<T, GB>(row, s_tot, s_tri, cnt, tri + (int64_t)j * GB);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < GB; ++t) hp[t] = s_h[t];
+    }
+    const T hn = Ar<T>::sqrt(s_tot[0]);
+    if (hn > T(0) && isfinite((double)hn)) {
+        const Quot<T> by(hn);
+        for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) z[r] = by(z[r]);
+    }
+    if (blockIdx.x == 0 && w == 0) {
+        if (lane == 0) {
+            tag_publish(hn, hq + (int64_t)(j + 1) * TagWords<T>::W, tag);
+            st->bar.seq = tag;
+        }
+        __syncwarp();
+        if (!givens_column<T>(j, kmax, H, cs, sn, g, st, hq, tag, tmo) && lane == 0) {
+            st->status = BSPAI_TIMEOUT;
+            st->done = 1;
         }
     }
 }
@@ -258,181 +242,149 @@ __global__ void __launch_bounds__(512) k_mgs(T* __restrict__ V, int64_t ldv, int
 constexpr int kMgsBlocks = 64;  // fewest blocks the on-chip MGS kernel is given
 // A block's bytes of one basis vector (at the instance's capacity) from which
 // an on-chip MGS instance polls its reductions by bulk copies
-// (tag_poll_warp_bulk) instead of loads.  Measured (fp32, 64-128 blocks,
-// 64-step GMRES runs): load polling 5 % faster at 4 KB per block
-// (n = 64,000), even at 7 KB; bulk polling 11 / 3 / 4 % faster at 16 / 32 /
-// 64 KB (n = 262,144 / 512,000 / 2,097,152); with 9 blocks per solve (16
-// right-hand sides side by side) and 29 KB per block, slower.  Instances whose
-// capacity is below the threshold are compiled without the bulk path (their
-// load poll's code unchanged); the others take it when the launch asks.
+// (tag_poll_row_bulk) instead of loads.  Measured (fp32, 64-128 blocks,
+// 64-step GMRES runs, one vector per reduction): load polling 5 % faster at
+// 4 KB per block (n = 64,000), even at 7 KB; bulk polling 11 / 3 / 4 % faster at
+// 16 / 32 / 64 KB (n = 262,144 / 512,000 / 2,097,152); with 9 blocks per solve
+// (16 right-hand sides side by side) and 29 KB per block, slower.  Instances
+// whose capacity is below the threshold are compiled without the bulk path;
+// the others take it when the launch asks.
 constexpr int64_t kBulkPollBytes = 16 * 1024;
 
-// The Givens block: with giv = 1 the last block of an on-chip MGS launch takes
-// no rows.  Its first warp reads every pass's total from the same tagged slots
-// as the other blocks (so the same values), applies rotation i - 1 of the
-// earlier steps to column j as soon as h_{i,j} has arrived -- while the other
-// blocks run the later passes -- and after the last pass forms the new
-// rotation, g and the tau test.  One thread's sweep over the earlier
-// rotations costs about 480 cycles per rotation on GB300's narrow fp64 pipe
-// (21 us at j = 90), and here it overlaps the passes instead of following the
-// last one.  Same operations in the same order as givens_step.
-template <typename T>
-__device__ void givens_block(int j, int kmax, double* H, double* cs, double* sn, double* g, GmresState* st,
-                             const unsigned long long* tags, int G, unsigned seq0, unsigned long long tmo) {
-    if (threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
-    double* __restrict__ hc = H + (int64_t)j * (kmax + 1);
-    double carry = 0.0;
-    T hz = T(0);
-    bool ok = true;
-    for (int i = 1; i <= j + 2; ++i) {
-        T h;
-        if (!tag_poll_warp<T>(tags, (i - 1) & 1, seq0 + (unsigned)i, G, &st->bar, tmo, &h)) {
-            ok = false;
-            break;
-        }
-        if (i == j + 2) {
-            hz = h;
-            break;
-        }
-        const int r = i - 1;  // h = h_{r,j}
-        if (lane == 0) {
-            if (r == 0) carry = (double)h;
-            else hc[r - 1] = givens_apply(cs[r - 1], sn[r - 1], carry, (double)h);
-        }
-    }
-    if (lane != 0) return;
-    if (!ok) {
-        st->status = BSPAI_TIMEOUT;
-        st->done = 1;
-        return;
-    }
-    // every block has read seq0 before its last partial, and this block read it
-    // at its start: advance it for the next launch
-    st->bar.seq = seq0 + (unsigned)j + 2u;
-    givens_finish(j, kmax, (double)Ar<T>::sqrt(hz), carry, hc, cs, sn, g, st);
-}
-
-// MGS step with the new vector z resident on chip: one block per SM owns a
-// contiguous range of rows, holds z for them in shared memory for all j + 2
-// passes, and streams each basis vector v_i exactly once (R rows per thread
-// of a BD-thread block, all loads of a pass issued before the thread waits on
-// the previous pass's reduction; BD = 512 for many rows per block, so that
-// the 2 R values a thread keeps stay in registers).  Per pass i: z <- z - h_{i-1} v_{i-1} (v_{i-1} kept in registers),
-// partial += v_i . z, arrive; the last pass forms ||z||_2 and writes v_{j+1}.
-// Same arithmetic as k_mgs (fp32 or fp64, no fused multiply-add).
-template <typename T, int R, int BD>
-__global__ void __launch_bounds__(BD, 1) k_mgs_res(T* __restrict__ V, int64_t ldv, int n, GmresState* st,
-                                                     double* H, double* cs, double* sn, double* g,
-                                                     unsigned long long* tags, unsigned long long tmo, int giv,
-                                                     int bulk) {
+// The on-chip MGS kernels: one block per SM owns a contiguous range of rows,
+// holds z for them for the whole step, and reads each basis vector once
+// (mgs.cuh).  With giv = 1 the last block of the launch takes no rows: its first
+// warp applies the earlier rotations to column j as the coefficients arrive,
+// while the other blocks run the later groups, and forms the new rotation, g and
+// the tau test after the last.  With giv = 0 the first block does so at the end.
+template <class I>
+__device__ __forceinline__ void mgs_kernel(typename I::type* __restrict__ V, int64_t ldv, int n, GmresState* st,
+                                           double* H, double* cs, double* sn, double* g, unsigned long long* tags,
+                                           unsigned long long* hq, void* tri, unsigned long long tmo, int giv,
+                                           int bulk) {
+    typedef typename I::type T;
     extern __shared__ __align__(16) unsigned char smraw[];
-    T* zs = reinterpret_cast<T*>(smraw);
-    constexpr bool kBulk = (int64_t)R * BD * (int64_t)sizeof(T) >= kBulkPollBytes;  // and bulk: the launch's choice
-    __shared__ T s_w[32];
-    __shared__ T s_tot;
+    __shared__ MgsShared<I> sh;
     __shared__ unsigned s_seq;
-    __shared__ int s_ok, s_j, s_done, s_kmax;
-    __shared__ __align__(16) unsigned long long s_slots[kBulk ? 2 * kTagMaxBlocks + 2 : 2];  // warp 0's copies
-    __shared__ __align__(8) uint64_t s_mbar;
-    unsigned phase = 0;
-    if (threadIdx.x == 0) {
+    __shared__ int s_j, s_done, s_kmax;
+    const int tid = threadIdx.x;
+    if (tid == 0) {
         s_j = st->j;
         s_done = st->done;
         s_kmax = st->kmax;
         s_seq = *(volatile unsigned*)&st->bar.seq;  // reductions of this launch are s_seq + 1, s_seq + 2, ...
-        if (kBulk) {
-            mbar_init(&s_mbar, 1);
-            mbar_init_fence();
-        }
+        mgs_shared_init<I>(sh);
     }
     __syncthreads();
     if (s_done) return;
     const int j = s_j, kmax = s_kmax;
-    const unsigned seq0 = s_seq;
+    const unsigned seq0 = s_seq, tag = seq0 + 1u;
+    const unsigned seq1 = seq0 + (unsigned)(j / I::GB) + 2u;  // the last reduction's number
     const int G = gridDim.x - giv;  // blocks that hold rows and publish partial sums
-    if (giv && blockIdx.x == G) {
-        givens_block<T>(j, kmax, H, cs, sn, g, st, tags, G, seq0, tmo);
-        return;
-    }
-    int64_t r0, r1;
-    block_rows(n, G, r0, r1);
-    const int nb = r1 > r0 ? (int)(r1 - r0) : 0;
-    const int tid = threadIdx.x;
-    constexpr int bd = BD;
-    T* z = V + (int64_t)(j + 1) * ldv + r0;
-    const T* v0 = V + r0;
-    T vcur[R], vnext[R];
+    const bool rotates = giv ? blockIdx.x == G : blockIdx.x == 0;
+    if (blockIdx.x < G) {
+        int64_t r0, r1;
+        block_rows(n, G, r0, r1);
+        MgsRows<I> R;
+        R.nb = r1 > r0 ? (int)(r1 - r0) : 0;
+        T* zg = V + (int64_t)(j + 1) * ldv + r0;
+        typename I::P z[I::NP];
+        unsigned char* zs = smraw + (size_t)I::S * I::stage_bytes;
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-        const int lr = tid + t * bd;
-        vcur[t] = T(0);
-        vnext[t] = T(0);
-        if (lr < nb) {
-            zs[lr] = z[lr];
-            vcur[t] = v0[lr];
-        }
-    }
-    T acc = T(0);
+        for (int u = 0; u < I::NU; ++u) {
+            if constexpr (I::ZS) {
+                typename I::P t[I::PN];
+                unit_load<I>(R, zg, u, t);
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-        const int lr = tid + t * bd;
-        if (lr < nb) acc = Ar<T>::add(acc, Ar<T>::mul(vcur[t], zs[lr]));
-    }
-    tag_arrive(acc, tags, 0, seq0 + 1u, s_w, G);
-    for (int i = 1; i <= j + 1; ++i) {
-        if (i <= j) {
-            const T* vi = V + (int64_t)i * ldv + r0;
-#pragma unroll
-            for (int t = 0; t < R; ++t) {
-                const int lr = tid + t * bd;
-                if (lr < nb) vnext[t] = vi[lr];
+                for (int k = 0; k < I::PN; ++k)
+                    reinterpret_cast<typename I::P*>(zs)[(tid + u * I::BD) * I::PN + k] = t[k];
+            } else {
+                unit_load<I>(R, zg, u, z + u * I::PN);
             }
         }
-        const T h = tag_wait_bulk(tags, (i - 1) & 1, seq0 + (unsigned)i, &st->bar, tmo, &s_tot, &s_ok, G, s_slots,
-                                  &s_mbar, phase, kBulk && bulk);
-        if (!s_ok) {
+        const MgsIo io{tags, hq, tri, &st->bar, tmo, G, bulk, blockIdx.x == 0, blockIdx.x == 0};
+        unsigned seq = seq0, phase = 0;
+        T hz;
+        if (!mgs_passes<I>(sh, io, R, z, smraw, zs, V + r0, ldv, j, tag, seq, phase, hz)) {
             if (blockIdx.x == 0 && tid == 0) {
                 st->status = BSPAI_TIMEOUT;
                 st->done = 1;
             }
             return;
         }
-        if (!giv && blockIdx.x == 0 && tid == 0) H[(int64_t)j * (kmax + 1) + (i - 1)] = (double)h;
-        acc = T(0);
+        const T hn = Ar<T>::sqrt(hz);
+        const bool norm = hn > T(0) && isfinite((double)hn);
+        const Quot<T> by(hn);
+        const int nu = R.units();
 #pragma unroll
-        for (int t = 0; t < R; ++t) {
-            const int lr = tid + t * bd;
-            if (lr < nb) {
-                const T zr = Ar<T>::sub(zs[lr], Ar<T>::mul(h, vcur[t]));
-                zs[lr] = zr;
-                acc = Ar<T>::add(acc, Ar<T>::mul(i <= j ? vnext[t] : zr, zr));
+        for (int u = 0; u < I::NU; ++u) {
+            if (u >= nu) break;
+            typename I::P t[I::PN];
+#pragma unroll
+            for (int k = 0; k < I::PN; ++k) {
+                if constexpr (I::ZS) t[k] = reinterpret_cast<typename I::P*>(zs)[(tid + u * I::BD) * I::PN + k];
+                else t[k] = z[u * I::PN + k];
+                if (norm) t[k] = pk_quot(t[k], by);
+            }
+            unit_store<I>(R, zg, u, t);
+        }
+    }
+    if (rotates && tid < 32) {
+        const bool ok = givens_column<T>(j, kmax, H, cs, sn, g, st, hq, tag, tmo);
+        if (tid == 0) {
+            if (ok) {
+                // every block has read seq0 (the reductions are complete): advance it
+                st->bar.seq = seq1;
+            } else {
+                st->status = BSPAI_TIMEOUT;
+                st->done = 1;
             }
         }
-        tag_arrive(acc, tags, i & 1, seq0 + (unsigned)i + 1u, s_w, G);
-#pragma unroll
-        for (int t = 0; t < R; ++t) vcur[t] = vnext[t];
     }
-    const T h2 = tag_wait_bulk(tags, (j + 1) & 1, seq0 + (unsigned)j + 2u, &st->bar, tmo, &s_tot, &s_ok, G, s_slots,
-                               &s_mbar, phase, kBulk && bulk);
-    if (!s_ok) {
-        if (blockIdx.x == 0 && tid == 0) {
-            st->status = BSPAI_TIMEOUT;
-            st->done = 1;
-        }
-        return;
-    }
-    // every block has read seq0 (its first slot carries seq0 + 1): advance it
-    // (with a Givens block, that block advances it: it may have started last)
-    if (!giv && blockIdx.x == 0 && tid == 0) st->bar.seq = seq0 + (unsigned)j + 2u;
-    const T hn = Ar<T>::sqrt(h2);
-    const bool norm = hn > T(0) && isfinite((double)hn);
-#pragma unroll
-    for (int t = 0; t < R; ++t) {
-        const int lr = tid + t * bd;
-        if (lr < nb) z[lr] = norm ? Ar<T>::div(zs[lr], hn) : zs[lr];
-    }
-    if (!giv && blockIdx.x == 0 && tid == 0) givens_step(j, kmax, (double)hn, H, cs, sn, g, st);
+}
+
+// rows of a thread one by one (R = 1) or in 16-byte units; fp64, and the smallest fp32 chunks
+template <typename T, int R, int BD>
+struct ResInst;
+template <>
+struct ResInst<float, 1, 1024> : MgsInst<float, 1, 1, 1024, 8, 16, false, false> {};
+template <>
+struct ResInst<double, 1, 1024> : MgsInst<double, 1, 1, 1024, 8, 16, false, false> {};
+template <>
+struct ResInst<double, 2, 1024> : MgsInst<double, 2, 1, 1024, 4, 8, true, false> {};
+template <>
+struct ResInst<double, 4, 1024> : MgsInst<double, 2, 2, 1024, 4, 5, true, false> {};
+template <>
+struct ResInst<double, 8, 1024> : MgsInst<double, 1, 8, 1024, 2, 2, true, true> {};
+template <typename T, int R, int BD>
+__global__ void __launch_bounds__(BD, 1) k_mgs_res(T* __restrict__ V, int64_t ldv, int n, GmresState* st, double* H,
+                                                   double* cs, double* sn, double* g, unsigned long long* tags,
+                                                   unsigned long long* hq, void* tri, unsigned long long tmo, int giv,
+                                                   int bulk) {
+    mgs_kernel<ResInst<T, R, BD>>(V, ldv, n, st, H, cs, sn, g, tags, hq, tri, tmo, giv, bulk);
+}
+
+// fp32, P pairs of adjacent rows per thread
+template <int P, int BD>
+struct ResInst2;
+template <>
+struct ResInst2<1, 1024> : MgsInst<float, 2, 1, 1024, 8, 16, false, false> {};
+template <>
+struct ResInst2<2, 1024> : MgsInst<float, 4, 1, 1024, 4, 8, true, false> {};
+template <>
+struct ResInst2<4, 1024> : MgsInst<float, 4, 2, 1024, 4, 6, true, false> {};
+template <>
+struct ResInst2<12, 512> : MgsInst<float, 4, 6, 512, 2, 4, true, false> {};
+template <>
+struct ResInst2<14, 512> : MgsInst<float, 4, 7, 512, 2, 3, true, false> {};
+template <>
+struct ResInst2<16, 512> : MgsInst<float, 4, 8, 512, 2, 3, true, false> {};
+template <int P, int BD>
+__global__ void __launch_bounds__(BD, 1) k_mgs_res2(float* __restrict__ V, int64_t ldv, int n, GmresState* st,
+                                                    double* H, double* cs, double* sn, double* g,
+                                                    unsigned long long* tags, unsigned long long* hq, void* tri,
+                                                    unsigned long long tmo, int giv, int bulk) {
+    mgs_kernel<ResInst2<P, BD>>(V, ldv, n, st, H, cs, sn, g, tags, hq, tri, tmo, giv, bulk);
 }
 
 // y = R^-1 g by column-oriented back substitution (fp64): for i = k-1 .. 0,
@@ -583,141 +535,6 @@ __global__ void k_absmax(int n, const double* __restrict__ v, double* __restrict
     block_atomic_max_nonneg(out, a);
 }
 
-// k_mgs_res for fp32 with the rows of a thread taken in adjacent pairs: every
-// multiply and add is a packed two-lane fp32 operation (each lane correctly
-// rounded, no fused multiply-add: the same arithmetic per element), z and the
-// basis rows move as float2, and the thread's partial sum is carried in two
-// lanes that are added at the end.  z stays in registers for all j + 2 passes
-// (2 P values per thread beside v_{i-1} and v_i: at most 128 registers for
-// P = 16 at 512 threads, no spills), so a pass touches no shared memory
-// outside its reduction: measured at 128^3 the pass fell from 3.53 to 3.31 us
-// against z held in shared memory.  P pairs per thread; the rows of a block
-// are its contiguous chunk (an even start, at most one unpaired last row).
-__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-
-template <int P, int BD>
-__global__ void __launch_bounds__(BD, 1) k_mgs_res2(float* __restrict__ V, int64_t ldv, int n, GmresState* st,
-                                                      double* H, double* cs, double* sn, double* g,
-                                                      unsigned long long* tags, unsigned long long tmo, int giv,
-                                                      int bulk) {
-    constexpr bool kBulk = (int64_t)2 * P * BD * (int64_t)sizeof(float) >= kBulkPollBytes;
-    __shared__ float s_w[32];
-    __shared__ float s_tot;
-    __shared__ unsigned s_seq;
-    __shared__ int s_ok, s_j, s_done, s_kmax;
-    __shared__ __align__(16) unsigned long long s_slots[kBulk ? 2 * kTagMaxBlocks + 2 : 2];  // warp 0's copies
-    __shared__ __align__(8) uint64_t s_mbar;
-    unsigned phase = 0;
-    if (threadIdx.x == 0) {
-        s_j = st->j;
-        s_done = st->done;
-        s_kmax = st->kmax;
-        s_seq = *(volatile unsigned*)&st->bar.seq;
-        if (kBulk) {
-            mbar_init(&s_mbar, 1);
-            mbar_init_fence();
-        }
-    }
-    __syncthreads();
-    if (s_done) return;
-    const int j = s_j, kmax = s_kmax;
-    const unsigned seq0 = s_seq;
-    const int G = gridDim.x - giv;  // blocks that hold rows and publish partial sums
-    if (giv && blockIdx.x == G) {
-        givens_block<float>(j, kmax, H, cs, sn, g, st, tags, G, seq0, tmo);
-        return;
-    }
-    int64_t r0, r1;
-    block_rows(n, G, r0, r1);
-    const int nb = r1 > r0 ? (int)(r1 - r0) : 0;
-    const int tid = threadIdx.x;
-    // pair q covers rows 2q, 2q + 1 of the chunk; the second may lie past nb
-    auto ld2 = [&](const float* p, int q) -> float2 {
-        if (2 * q + 1 < nb) return *reinterpret_cast<const float2*>(p + 2 * q);
-        return make_float2(p[2 * q], 0.0f);
-    };
-    float* z = V + (int64_t)(j + 1) * ldv + r0;
-    const float* v0 = V + r0;
-    // z (this thread's rows of the new vector), v_{i-1} and v_i in registers
-    float2 zr[P], vcur[P], vnext[P];
-    const float2 zero2 = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int t = 0; t < P; ++t) {
-        const int q = tid + t * BD;
-        zr[t] = zero2;
-        vcur[t] = zero2;
-        vnext[t] = zero2;
-        if (2 * q < nb) {
-            zr[t] = ld2(z, q);
-            vcur[t] = ld2(v0, q);
-        }
-    }
-    float2 acc2 = zero2;
-#pragma unroll
-    for (int t = 0; t < P; ++t) {
-        const int q = tid + t * BD;
-        if (2 * q < nb) acc2 = __fadd2_rn(acc2, __fmul2_rn(vcur[t], zr[t]));
-    }
-    tag_arrive(__fadd_rn(acc2.x, acc2.y), tags, 0, seq0 + 1u, s_w, G);
-    for (int i = 1; i <= j + 1; ++i) {
-        if (i <= j) {
-            const float* vi = V + (int64_t)i * ldv + r0;
-#pragma unroll
-            for (int t = 0; t < P; ++t) {
-                const int q = tid + t * BD;
-                if (2 * q < nb) vnext[t] = ld2(vi, q);
-            }
-        }
-        const float h = tag_wait_bulk(tags, (i - 1) & 1, seq0 + (unsigned)i, &st->bar, tmo, &s_tot, &s_ok, G,
-                                      s_slots, &s_mbar, phase, kBulk && bulk);
-        if (!s_ok) {
-            if (blockIdx.x == 0 && tid == 0) {
-                st->status = BSPAI_TIMEOUT;
-                st->done = 1;
-            }
-            return;
-        }
-        if (!giv && blockIdx.x == 0 && tid == 0) H[(int64_t)j * (kmax + 1) + (i - 1)] = (double)h;
-        const float2 h2 = make_float2(h, h);
-        acc2 = zero2;
-#pragma unroll
-        for (int t = 0; t < P; ++t) {
-            const int q = tid + t * BD;
-            if (2 * q < nb) {
-                zr[t] = f2_sub(zr[t], __fmul2_rn(h2, vcur[t]));
-                acc2 = __fadd2_rn(acc2, __fmul2_rn(i <= j ? vnext[t] : zr[t], zr[t]));
-            }
-        }
-        tag_arrive(__fadd_rn(acc2.x, acc2.y), tags, i & 1, seq0 + (unsigned)i + 1u, s_w, G);
-#pragma unroll
-        for (int t = 0; t < P; ++t) vcur[t] = vnext[t];
-    }
-    const float hz = tag_wait_bulk(tags, (j + 1) & 1, seq0 + (unsigned)j + 2u, &st->bar, tmo, &s_tot, &s_ok, G,
-                                   s_slots, &s_mbar, phase, kBulk && bulk);
-    if (!s_ok) {
-        if (blockIdx.x == 0 && tid == 0) {
-            st->status = BSPAI_TIMEOUT;
-            st->done = 1;
-        }
-        return;
-    }
-    // (with a Givens block, that block advances it: it may have started last)
-    if (!giv && blockIdx.x == 0 && tid == 0) st->bar.seq = seq0 + (unsigned)j + 2u;
-    const float hn = __fsqrt_rn(hz);
-    const bool norm = hn > 0.0f && isfinite((double)hn);
-#pragma unroll
-    for (int t = 0; t < P; ++t) {
-        const int q = tid + t * BD;
-        if (2 * q < nb) {
-            float2 zo = zr[t];
-            if (norm) zo = make_float2(__fdiv_rn(zo.x, hn), __fdiv_rn(zo.y, hn));
-            if (2 * q + 1 < nb) *reinterpret_cast<float2*>(z + 2 * q) = zo;
-            else z[2 * q] = zo.x;
-        }
-    }
-    if (!giv && blockIdx.x == 0 && tid == 0) givens_step(j, kmax, (double)hn, H, cs, sn, g, st);
-}
-
 // ---------------------------------------------------------------- host side
 struct HostFlags {
     int j, done, status, kmax;
@@ -731,8 +548,11 @@ struct GmresWork {
     int64_t ldv = 0;
     void* V = nullptr;
     void* w = nullptr;
-    void* part = nullptr;
-    unsigned long long* tags = nullptr;  // k_mgs_res slots: 2 parities x blocks x 2 words
+    unsigned char* aux = nullptr;        // the reductions' buffers (carve):
+    unsigned long long* tags = nullptr;  //   tagged slots: 2 parities x kMgsMaxVals x kTagMaxBlocks x 2 words
+    unsigned long long* hq = nullptr;    //   tagged coefficients of the current column
+    void* tri = nullptr;                 //   the groups' (I + L)^-1, up to kMgsMaxVals / 2 values per basis vector
+    void* part = nullptr;                //   partial sums of the grid-barrier reductions
     GmresState* st = nullptr;
     double *H = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr, *norms = nullptr;
     HostFlags* hflags = nullptr;  // pinned
@@ -749,7 +569,31 @@ struct GmresWork {
     size_t res_smem = 0;
     cudaStream_t s = nullptr;
 
-    static size_t tag_words() { return (size_t)4 * kTagMaxBlocks; }
+    // tags and hq, which must start at zero (the sequence numbers that tag them start at one)
+    size_t tagged_bytes() const {
+        return sizeof(unsigned long long) * ((size_t)2 * kMgsMaxVals * kTagMaxBlocks * 2 + 2 * ((size_t)kmax + 2));
+    }
+    size_t aux_bytes() const {
+        const size_t es = ug == BSPAI_FP64 ? 8 : 4;
+        return tagged_bytes() + es * (kMgsMaxVals / 2) * ((size_t)kmax + 1) + es * 2 * kMgsMaxVals * (size_t)G;
+    }
+    // the rows past n of every basis vector: the on-chip MGS kernels copy whole 16-byte units
+    int zero_pad() const {
+        const size_t es = ug == BSPAI_FP64 ? 8 : 4;
+        const int64_t to = ceil_div(n, 4) * 4;
+        if (to == n) return BSPAI_OK;
+        CUDA_TRY(cudaMemset2DAsync(static_cast<unsigned char*>(V) + es * (size_t)n, es * (size_t)ldv, 0,
+                                   es * (size_t)(to - n), (size_t)kmax + 1, s));
+        return BSPAI_OK;
+    }
+    void carve(void* base) {
+        const size_t es = ug == BSPAI_FP64 ? 8 : 4;
+        aux = static_cast<unsigned char*>(base);
+        tags = reinterpret_cast<unsigned long long*>(aux);
+        hq = tags + (size_t)2 * kMgsMaxVals * kTagMaxBlocks * 2;
+        tri = aux + tagged_bytes();
+        part = static_cast<unsigned char*>(tri) + es * (kMgsMaxVals / 2) * ((size_t)kmax + 1);
+    }
     int sms = 0;  // SMs the cooperative kernels may use (one block of k_mgs_res each)
     int alloc(int n_, int kmax_, int ug_, int up_, double timeout_s, int max_blocks, cudaStream_t st_) {
         sms = max_blocks > 0 && max_blocks < num_sms() ? max_blocks : num_sms();
@@ -779,9 +623,10 @@ struct GmresWork {
         G = (occ >= 2 ? 2 : 1) * sms;
         BSPAI_TRY(dalloc(&V, es * (size_t)ldv * (size_t)(kmax + 1), s));
         BSPAI_TRY(dalloc(&w, es * (size_t)ldv, s));
-        BSPAI_TRY(dalloc(&part, es * 2 * (size_t)G, s));
-        BSPAI_TRY(dalloc_t(&tags, tag_words(), s));
-        CUDA_TRY(cudaMemsetAsync(tags, 0, sizeof(unsigned long long) * tag_words(), s));
+        BSPAI_TRY(dalloc_t(&aux, aux_bytes(), s));
+        carve(aux);
+        CUDA_TRY(cudaMemsetAsync(aux, 0, tagged_bytes(), s));
+        BSPAI_TRY(zero_pad());
         BSPAI_TRY(dalloc_t(&st, 1, s));
         BSPAI_TRY(dalloc_t(&H, (size_t)(kmax + 1) * kmax, s));
         BSPAI_TRY(dalloc_t(&cs, (size_t)kmax + 1, s));
@@ -798,10 +643,11 @@ struct GmresWork {
         return choose_mgs(*this);
     }
     void release() {
-        dfree(V, s); dfree(w, s); dfree(part, s); dfree(tags, s); dfree(st, s); dfree(H, s); dfree(cs, s);
+        dfree(V, s); dfree(w, s); dfree(aux, s); dfree(st, s); dfree(H, s); dfree(cs, s);
         dfree(sn, s); dfree(g, s); dfree(y, s); dfree(norms, s);
-        V = w = part = nullptr;
-        tags = nullptr;
+        V = w = part = tri = nullptr;
+        aux = nullptr;
+        tags = hq = nullptr;
         st = nullptr;
         H = cs = sn = g = y = norms = nullptr;
     }
@@ -809,79 +655,96 @@ struct GmresWork {
 
 // One k_mgs_res / k_mgs_res2 instance: its kernel, kind (1: k_mgs_res, rows of a
 // thread one by one; 2: k_mgs_res2, rows in packed pairs), rows (R) or pairs (P)
-// per thread, and block size.  The instance is the smallest that holds a
-// block's chunk of rows: every instance listed here is reachable from
-// choose_mgs for some order n (the parity tests run each one).
+// per thread, block size and dynamic shared memory.  The instance is the
+// smallest that holds a block's chunk of rows: every instance listed here is
+// reachable from choose_mgs for some order n (the parity tests run each one).
 struct ResInstance {
     void* fn = nullptr;
     int kind = 0, per_thread = 0, bd = 0;
+    size_t smem = 0;
 };
+
+template <typename T, int R, int BD>
+static ResInstance res_instance() {
+    return {(void*)k_mgs_res<T, R, BD>, 1, R, BD, ResInst<T, R, BD>::smem};
+}
+template <int P, int BD>
+static ResInstance res_instance2() {
+    return {(void*)k_mgs_res2<P, BD>, 2, P, BD, ResInst2<P, BD>::smem};
+}
 
 template <typename T>
 static ResInstance pick_res(int64_t chunk) {
     const int R = (int)ceil_div(chunk, 1024);
-    if (R <= 1) return {(void*)k_mgs_res<T, 1, 1024>, 1, 1, 1024};
+    if (R <= 1) return res_instance<T, 1, 1024>();
     if constexpr (sizeof(T) == 4) {
         // fp32: rows in adjacent pairs, packed two-lane arithmetic
-        if (R <= 2) return {(void*)k_mgs_res2<1, 1024>, 2, 1, 1024};
-        if (R <= 4) return {(void*)k_mgs_res2<2, 1024>, 2, 2, 1024};
-        if (R <= 8) return {(void*)k_mgs_res2<4, 1024>, 2, 4, 1024};
+        if (R <= 2) return res_instance2<1, 1024>();
+        if (R <= 4) return res_instance2<2, 1024>();
+        if (R <= 8) return res_instance2<4, 1024>();
         // more rows per block: 512 threads with more pairs each (chunk > 8192)
         const int Rp = (int)ceil_div(chunk, 512);
-        if (Rp <= 24) return {(void*)k_mgs_res2<12, 512>, 2, 12, 512};
-        if (Rp <= 28) return {(void*)k_mgs_res2<14, 512>, 2, 14, 512};
-        if (Rp <= 32) return {(void*)k_mgs_res2<16, 512>, 2, 16, 512};
+        if (Rp <= 24) return res_instance2<12, 512>();
+        if (Rp <= 28) return res_instance2<14, 512>();
+        if (Rp <= 32) return res_instance2<16, 512>();
         return {};
     } else {
-        // fp64: z in shared memory, at most 8192 rows of a block (64 KB)
-        if (R <= 2) return {(void*)k_mgs_res<T, 2, 1024>, 1, 2, 1024};
-        if (R <= 4) return {(void*)k_mgs_res<T, 4, 1024>, 1, 4, 1024};
-        if (R <= 8) return {(void*)k_mgs_res<T, 8, 1024>, 1, 8, 1024};
+        if (R <= 2) return res_instance<T, 2, 1024>();
+        if (R <= 4) return res_instance<T, 4, 1024>();
+        if (R <= 8) return res_instance<T, 8, 1024>();
         return {};
     }
 }
 
 // Use the on-chip MGS kernel when one block per SM can hold its rows of z on
-// chip (fp32: in registers; fp64: in shared memory, at most 200 KB) with at
-// most 32 (fp32) / 16 (fp64) rows per thread of a 512-thread block.
+// chip: at most 16,384 rows of a block in fp32, 8,192 in fp64.
 static int choose_mgs(GmresWork& W) {
     W.res_fn = nullptr;
     // As few blocks as hold the rows of z on chip, but not fewer than kMgsBlocks: each
-    // grid reduction of the j + 2 per Arnoldi step waits for every block, and fewer
-    // blocks shorten it (measured per pass, n = 65,536 / 262,144: 2.5 / 3.1 us at 152
-    // blocks, 1.6 / 1.9 us at 64) while one block still streams its rows faster than
-    // the reduction completes.
-    // rows per block of the largest instance.  At 128^3 fewer blocks stopped paying: 103
-    // blocks of 40 fp32 rows per thread solved in 90.8 ms against 87.7 ms at 128 blocks of
-    // 32 (the longer per-block update outweighs the shorter reduction), and a scalar
-    // 768-thread instance (22,272 rows, register spills) took 107.6 ms at 95 blocks.
+    // grid reduction waits for every block, and fewer blocks shorten it (measured per
+    // reduction, n = 65,536 / 262,144: 2.5 / 3.1 us at 152 blocks, 1.6 / 1.9 us at 64).
+    // At 128^3 fewer blocks stopped paying: 103 blocks of 40 fp32 rows per thread solved
+    // in 90.8 ms against 87.7 ms at 128 blocks of 32, and a scalar 768-thread instance
+    // (22,272 rows, register spills) took 107.6 ms at 95 blocks.
     const int64_t cap = W.ug == BSPAI_FP64 ? 8192 : 16384;
     int Gr = (int)ceil_div(W.n, cap);
     if (Gr < kMgsBlocks) Gr = kMgsBlocks;
-    if (Gr > W.sms) Gr = W.sms;
+    // the Givens block wants an SM of its own (one block per SM at these sizes): the
+    // rotations of a column otherwise follow its last reduction
+    if (Gr >= W.sms) Gr = W.sms > 1 && ceil_div(W.n, W.sms - 1) <= cap ? W.sms - 1 : W.sms;
     if (Gr > kTagMaxBlocks) return BSPAI_OK;
-    const int64_t chunk = ceil_div(ceil_div(W.n, Gr), 32) * 32;
+    int64_t chunk = ceil_div(ceil_div(W.n, Gr), 32) * 32;
     const size_t es = W.ug == BSPAI_FP64 ? 8 : 4;
-    const size_t smem = (size_t)chunk * es;
-    if (smem > 200 * 1024) return BSPAI_OK;
     const ResInstance ri = es == 8 ? pick_res<double>(chunk) : pick_res<float>(chunk);
     if (!ri.fn) return BSPAI_OK;
-    CUDA_TRY(cudaFuncSetAttribute(ri.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (es == 8 && ri.per_thread > 1) {
+        // fp64 is bound by the narrow fp64 pipe of the SMs that hold rows: spread the rows
+        // over more blocks, down to just over half of the instance's capacity (per vector
+        // at n = 262,144: 9.0 us before, 3.6 with groups of 4 on 127 blocks)
+        const int64_t least = (int64_t)ri.per_thread * ri.bd / 2 + 32;
+        const int spare = W.sms - 1 > 0 ? W.sms - 1 : 1;
+        int64_t c = ceil_div(ceil_div(W.n, spare < kTagMaxBlocks ? spare : kTagMaxBlocks), 32) * 32;
+        if (c < least) c = least;
+        if (c < chunk) {
+            chunk = c;
+            Gr = (int)ceil_div(W.n, chunk);
+        }
+    }
+    CUDA_TRY(cudaFuncSetAttribute(ri.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ri.smem));
     int occ = 0;
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ri.fn, ri.bd, smem));
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ri.fn, ri.bd, ri.smem));
     if (occ < 1) return BSPAI_OK;
     W.res_fn = ri.fn;
     W.res_bd = ri.bd;
     W.res_kind = ri.kind;
     W.res_per_thread = ri.per_thread;
     W.Gr = Gr;
-    // the Givens block needs an SM of its own (one block per SM at these sizes)
     W.giv = Gr + 1 <= W.sms ? 1 : 0;
     // bulk-copy polling where it was measured to pay: at least kMgsBlocks blocks (a solve
     // confined to a few SMs, as each of several concurrent right-hand sides is, polls few
     // slots and the copy engine's round trip loses) and kBulkPollBytes of a vector per block
     W.bulk = Gr >= kMgsBlocks && (int64_t)chunk * (int64_t)es >= kBulkPollBytes ? 1 : 0;
-    W.res_smem = smem;
+    W.res_smem = ri.smem;
     return BSPAI_OK;
 }
 
@@ -952,11 +815,12 @@ static int gmres_run(GmresWork& W, const bspai_matrix* A, const bspai_bucketed* 
                 int nn = n;
                 int64_t ld = W.ldv;
                 if (W.res_fn) {
-                    void* args[] = {&V, &ld, &nn, &W.st, &W.H, &W.cs, &W.sn, &W.g, &W.tags, &W.tmo_ns, &W.giv,
-                                    &W.bulk};
+                    void* args[] = {&V, &ld, &nn, &W.st, &W.H, &W.cs, &W.sn, &W.g, &W.tags, &W.hq, &W.tri,
+                                    &W.tmo_ns, &W.giv, &W.bulk};
                     BSPAI_TRY(coop_launch_cfg(W.res_fn, W.Gr + W.giv, W.res_bd, W.res_smem, args, s));
                 } else {
-                    void* args[] = {&V, &ld, &nn, &W.st, &W.H, &W.cs, &W.sn, &W.g, &part, &W.tmo_ns};
+                    T* tri = reinterpret_cast<T*>(W.tri);
+                    void* args[] = {&V, &ld, &nn, &W.st, &W.H, &W.cs, &W.sn, &W.g, &part, &tri, &W.hq, &W.tmo_ns};
                     BSPAI_TRY(coop_launch((void*)k_mgs<T>, W.G, args, s));
                 }
             }
@@ -992,9 +856,9 @@ static int gmres_run(GmresWork& W, const bspai_matrix* A, const bspai_bucketed* 
     out.xmax = hn[1];
     if (hs.status == BSPAI_TIMEOUT) {
         // the barrier state is undefined after a timeout: reset it (and the
-        // tagged slots, whose numbers restart with it) for reuse
+        // tagged words, whose numbers restart with it) for reuse
         CUDA_TRY(cudaMemsetAsync(&W.st->bar, 0, sizeof(GridBar), s));
-        CUDA_TRY(cudaMemsetAsync(W.tags, 0, sizeof(unsigned long long) * GmresWork::tag_words(), s));
+        CUDA_TRY(cudaMemsetAsync(W.aux, 0, W.tagged_bytes(), s));
         return set_error(BSPAI_TIMEOUT, "gmres: a grid barrier exceeded its time limit");
     }
     return BSPAI_OK;
@@ -1429,8 +1293,10 @@ int bspai_gmres_b(bspai_A_h A, bspai_BM_h A_bucketed, bspai_BM_h BM, const doubl
 // process exits.
 namespace bspai {
 
-constexpr size_t kNoallocScratchBytes = 64ull << 20;  // 64 MiB
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+constexpr size_t kNoallocScratchBytes = 64ull << 20;  // 64 MiB: what a call's problem may take
+// beside it, the reductions' buffers (GmresWork::carve) at kmax = kKmaxLimit and any grid
+constexpr size_t kNoallocAuxBytes = 1ull << 20;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes + kNoallocAuxBytes];
 
 static std::mutex g_noalloc_mu;
 // Device address of the scratch per device ordinal, with the id of the CUDA
@@ -1539,7 +1405,7 @@ int bspai_gmres_noalloc(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_
     size_t sz[11] = {es * (size_t)W.ldv * (kx + 1), es * (size_t)W.ldv, es * 2 * (size_t)W.G, sizeof(GmresState),
                      sizeof(double) * (kx + 1) * kx, sizeof(double) * (kx + 1), sizeof(double) * (kx + 1),
                      sizeof(double) * (kx + 2), sizeof(double) * (kx + 1), sizeof(double) * 4,
-                     sizeof(unsigned long long) * GmresWork::tag_words()};
+                     sizeof(unsigned long long) * 4 * kTagMaxBlocks};
     off[0] = 0;
     for (int i = 0; i < 11; ++i) off[i + 1] = align256(off[i] + sz[i]);
     if (off[11] > kNoallocScratchBytes)
@@ -1551,7 +1417,6 @@ int bspai_gmres_noalloc(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_
     BSPAI_TRY(noalloc_scratch_address(reinterpret_cast<void**>(&base)));
     W.V = base + off[0];
     W.w = base + off[1];
-    W.part = base + off[2];
     W.st = reinterpret_cast<GmresState*>(base + off[3]);
     W.H = reinterpret_cast<double*>(base + off[4]);
     W.cs = reinterpret_cast<double*>(base + off[5]);
@@ -1559,7 +1424,10 @@ int bspai_gmres_noalloc(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_
     W.g = reinterpret_cast<double*>(base + off[7]);
     W.y = reinterpret_cast<double*>(base + off[8]);
     W.norms = reinterpret_cast<double*>(base + off[9]);
-    W.tags = reinterpret_cast<unsigned long long*>(base + off[10]);
+    if (W.aux_bytes() > kNoallocAuxBytes)
+        return set_error(BSPAI_ERR_INVALID, "bspai_gmres_noalloc: the reductions' buffers need %zu bytes",
+                         W.aux_bytes());
+    W.carve(base + kNoallocScratchBytes);
     static thread_local HostFlags t_flags;  // ordinary host memory
     W.hflags = &t_flags;
     BSPAI_TRY(choose_mgs(W));
@@ -1567,7 +1435,8 @@ int bspai_gmres_noalloc(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_
     // that must start at zero (solver state with its grid barrier, g, the
     // tagged slots that the barrier's sequence numbers restart with)
     CUDA_TRY(cudaMemsetAsync(W.st, 0, sizeof(GmresState), s));
-    CUDA_TRY(cudaMemsetAsync(W.tags, 0, sizeof(unsigned long long) * GmresWork::tag_words(), s));
+    CUDA_TRY(cudaMemsetAsync(W.aux, 0, W.tagged_bytes(), s));
+    BSPAI_TRY(W.zero_pad());
     CUDA_TRY(cudaMemsetAsync(W.g, 0, sizeof(double) * (kx + 2), s));
     GmresResult gr;
     int rc = u_g == BSPAI_FP64 ? gmres_run<double>(W, A, BM, r, o.tau, nullptr, d, gr)
