@@ -498,12 +498,13 @@ typedef struct {
 
 /* A schedule of the batched GMRES launch.  For a given block_threads every
  * schedule computes the same bits (the dot products of MGS are summed per
- * thread over rows t, t + block_threads, ... and then over the CTA in a fixed
- * tree); the other three fields move loads and storage only.
+ * thread over the 16-byte units t, t + block_threads, ... of its rows and then
+ * over the CTA in a fixed tree); the other three fields move loads and storage only.
  *   block_threads  CTA size: 128, 256 or 512 (one CTA per (system, RHS) pair).
- *   mgs_rows       the MGS load tile: rows per thread whose loads one pass
- *                  issues before any arithmetic (u_g fp32: 8 or 16; fp64: 4 or
- *                  8; 0 = the smaller).
+ *   mgs_rows       the MGS load tile (u_g fp32: 8 or 16; fp64: 4 or 8; 0 = the
+ *                  smaller): the smaller has one 16-byte unit of z and of each
+ *                  vector of two groups of four basis vectors in flight per
+ *                  thread, the larger two such units.
  *   z_shared_rows  pairs of at most this many rows keep z, the vector being
  *                  orthogonalised, in shared memory for the whole Arnoldi step
  *                  (0 = never; -1 = as many rows as fit); limited by the

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "mgs.cuh"
 #include "spmv_row.cuh"
 #include "tags.cuh"
 
@@ -36,25 +37,6 @@ namespace bspai {
 
 int launch_residual_batch(const bspai_matrix* A, int nrhs, const double* X, const double* Bv, double* R,
                           const int32_t* slice_seg, int nsys, double* prmax, double* pxmax, cudaStream_t s);
-
-template <typename T>
-struct BAr;
-template <>
-struct BAr<float> {
-    static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-    static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-    static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-    static __device__ __forceinline__ float div(float a, float b) { return __fdiv_rn(a, b); }
-    static __device__ __forceinline__ float sqrt(float a) { return __fsqrt_rn(a); }
-};
-template <>
-struct BAr<double> {
-    static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
-    static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
-    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
-    static __device__ __forceinline__ double div(double a, double b) { return __ddiv_rn(a, b); }
-    static __device__ __forceinline__ double sqrt(double a) { return __dsqrt_rn(a); }
-};
 
 // CTA-wide sum, identical in every thread (fixed reduction tree)
 template <typename T>
@@ -94,26 +76,25 @@ __device__ __forceinline__ double block_max(double v, double* s_w) {
     return r;
 }
 
-// Givens rotations on column j of H, update of g, tau test (fp64); thread 0
-__device__ void givens_pair(int j, int kmax, double hn, double* H, double* cs, double* sn, double* g, double tau,
-                            double beta, double* res, int* done) {
+// Givens rotations on column j of H (h_{0..j,j} as MGS left them, hn = h_{j+1,j}),
+// update of g, tau test (fp64); one warp, results in lane 0
+__device__ __forceinline__ void givens_pair(GivensBatch& gb, int j, int kmax, double hn, double* H, double* cs,
+                                            double* sn, double* g, double tau, double beta, double* res, int* done) {
+    const int lane = threadIdx.x & 31;
     double* __restrict__ hc = H + (int64_t)j * (kmax + 1);
-    const double* __restrict__ c_ = cs;
-    const double* __restrict__ s_ = sn;
-    hc[j + 1] = hn;
-    // the previous rotations applied to the new column; the entry each rotation hands
-    // to the next stays in a register, so only the running value is a dependent chain
-    // (the stored coefficients and column entries are independent loads)
-    double carry = j > 0 ? hc[0] : 0.0;
-    for (int i = 0; i < j; ++i) {
-        const double ci = c_[i], si = s_[i], hi1 = hc[i + 1];
-        const double t1 = __dadd_rn(__dmul_rn(ci, carry), __dmul_rn(si, hi1));
-        const double t2 = __dadd_rn(__dmul_rn(-si, carry), __dmul_rn(ci, hi1));
-        hc[i] = t1;
-        carry = t2;
+    double carry = 0.0;
+    for (int base = 0; base <= j; base += 32) {
+        const int i = base + lane;
+        const bool in = i <= j, rot = in && i >= 1;
+        const double hv = in ? hc[i] : 0.0, ci = rot ? cs[i - 1] : 1.0, si = rot ? sn[i - 1] : 0.0;
+        const int nin = j + 1 - base < 32 ? j + 1 - base : 32;
+        double met = 0.0;
+        if (base == 0) carry = __shfl_sync(0xffffffffu, hv, 0);
+        givens_chain(gb, base == 0 ? 1 : 0, nin, ci, si, hv, carry, met);
+        if (rot) hc[i - 1] = givens_entry(ci, si, hv, met);
     }
-    if (j > 0) hc[j] = carry;
-    const double a = hc[j], b = hc[j + 1];
+    if (lane != 0) return;
+    const double a = carry, b = hn;
     const double rr = __dsqrt_rn(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b)));
     double c = 1.0, s = 0.0;
     if (rr != 0.0) {
@@ -124,15 +105,16 @@ __device__ void givens_pair(int j, int kmax, double hn, double* H, double* cs, d
     sn[j] = s;
     hc[j] = rr;
     hc[j + 1] = 0.0;
-    g[j + 1] = __dmul_rn(-s, g[j]);
-    g[j] = __dmul_rn(c, g[j]);
-    *res = fabs(g[j + 1]);
-    const bool fin = isfinite(*res) && isfinite(hn) && isfinite(rr);
-    *done = (*res <= __dmul_rn(tau, beta)) || hn == 0.0 || j + 1 >= kmax || !fin;
+    const double gj = g[j], gn = __dmul_rn(-s, gj);
+    g[j + 1] = gn;
+    g[j] = __dmul_rn(c, gj);
+    *res = fabs(gn);
+    const bool fin = isfinite(gn) && isfinite(hn) && isfinite(rr);
+    *done = (fabs(gn) <= __dmul_rn(tau, beta)) || hn == 0.0 || j + 1 >= kmax || !fin;
 }
 
 // y[lr] = (M x)_{r0 + lr} for the rows of one system, under a bucket schedule
-// (kept out of line: the kernel calls it three times).
+// (kept out of line: the kernel calls it three times; M lies in shared memory).
 //   MS 0, row-fused: the CTA's threads stride over the rows, two rows per
 //     thread at a time (lr and lr + blockDim.x: two independent gather chains),
 //     each row through every bucket in turn.
@@ -180,13 +162,167 @@ __device__ __noinline__ void rows_apply(const BMDev& M, int r0, int ns, const XT
     if (lr < ns) y[lr] = from_f64<YT>(bucketed_row<XT>(M, r0 + lr, x));
 }
 
-// The MGS load tile: rows per thread whose loads a pass issues together (two
-// candidates per u_g for the autotuner)
+// Asks for a pair's part of a matrix in L2 ahead of its product (one warp, lane k for
+// bucket k): between two products of the step the basis has passed through L2, and a
+// row's chain of loads would otherwise wait for HBM at each link.
+__device__ __forceinline__ void ask_rows(const BMDev& M, int r0, int ns) {
+    const int k = threadIdx.x & 31;
+    if (k >= M.q || ns <= 0) return;
+    const BucketDev& B = M.b[k];
+    const int vb = B.prec == BSPAI_FP64 ? 8 : B.prec == BSPAI_FP32 ? 4 : B.prec == BSPAI_E4M3 ? 1 : 2;
+    const int64_t s0 = r0 >> 5, s1 = (r0 + ns) >> 5;
+    const int64_t p0 = __ldg(B.sptr + s0), slots = __ldg(B.sptr + s1) - p0;
+    // whole slices: 128 bytes of columns and at least 32 of values per slot of a row, and
+    // allocations are aligned, so both ends keep the engine's 16-byte rule
+    if (slots > 0) {
+        bulk_prefetch_l2(B.col + p0, (unsigned)(slots * 4));
+        bulk_prefetch_l2(static_cast<const unsigned char*>(B.val) + p0 * vb, (unsigned)(slots * vb));
+    }
+}
+
+// The MGS load tile of the pairs that are streamed (two candidates per u_g for the
+// autotuner): the smaller has one 16-byte unit of z and of two vector groups in flight
+// per thread, the larger two
 template <typename T>
 struct MgsU {
     static constexpr int lo = sizeof(T) == 4 ? 8 : 4;
     static constexpr int hi = 2 * lo;
 };
+
+// ------------------------------------------------------------------ MGS of a pair
+// Groups of four basis vectors (mgs.cuh) streamed from memory, pass g taking group
+// g - 1 out of z and forming the products with group g in one sweep, group g + 1
+// asked into L2 meanwhile.  Each thread owns the 16-byte units tid, tid + bd, ... and
+// adds their rows in that order, U / 8 (fp64: U / 4) units' loads ahead, so neither
+// the tile nor z's place changes a bit.  Returns h_{j+1,j} (in every thread); v_{j+1}
+// is written to its place in V.
+//
+// Bound by what one SM keeps in flight of the basis: 2.5 vector streams per basis
+// vector in 16-byte loads, one reduction per four, where one vector at a time took
+// four streams in 4-byte loads and a reduction each.  Whole solves of 384 pairs, ms
+// (one vector at a time -> this): orders 1,000 to 16,000 183 -> 108, 1,000 10.8 -> 6.8,
+// 15,500 554 -> 328; 160 pairs of 31,500 1,074 -> 729, 152 of 62,000 3,445 -> 2,136.
+// Groups of eight: 139 on the mixed orders (its registers spill), 1,798 at 62,000.
+// z and two vectors held on chip for a whole step (the single-system form on one SM)
+// lost to this at every order: 145 on the mixed ones.
+template <typename T>
+struct StreamShared {
+    T w[8][32], tot[8], h[4], tri[4][4];
+};
+template <typename T, int U>
+__device__ __noinline__ T stream_mgs(StreamShared<T>& sh, T* V, int64_t ldv, int ns, int j, T* z, double* hcol,
+                                     T* tri) {
+    constexpr int GB = 4, VW = 16 / (int)sizeof(T), RT = U / MgsU<T>::lo;
+    union Unit {
+        uint4 q;
+        T x[VW];
+    };
+    const int tid = threadIdx.x, bd = blockDim.x, lane = tid & 31, w = tid >> 5;
+    const int ng = j / GB + 1, nu = ns / VW;  // ns is a multiple of 32
+    T hp[GB];
+#pragma unroll
+    for (int t = 0; t < GB; ++t) hp[t] = T(0);
+    for (int gi = 0; gi <= ng; ++gi) {
+        const int i0 = gi * GB;
+        const bool last = gi == ng - 1, norm = gi == ng;
+        const int cnt = norm ? 0 : last ? j - i0 + 1 : GB;
+        const int have = gi > 0 ? (norm ? j + 1 - (i0 - GB) : GB) : 0;  // vectors of the previous group
+        if (tid < GB && i0 + GB + tid <= j)
+            bulk_prefetch_l2(V + (int64_t)(i0 + GB + tid) * ldv, (unsigned)(ns * (int)sizeof(T)));
+        T a[GB], q[GB], zz = T(0);
+#pragma unroll
+        for (int t = 0; t < GB; ++t) a[t] = q[t] = T(0);
+        for (int b0 = tid; b0 < nu; b0 += bd * RT) {
+            Unit zr[RT], pv[RT][GB], v[RT][GB];
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                const int u = b0 + r * bd;
+                const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+                zr[r].q = u < nu ? reinterpret_cast<const uint4*>(z)[u] : zero;
+#pragma unroll
+                for (int t = 0; t < GB; ++t) {
+                    pv[r][t].q = (t < have && u < nu)
+                                     ? reinterpret_cast<const uint4*>(V + (int64_t)(i0 - GB + t) * ldv)[u] : zero;
+                    v[r][t].q = (t < cnt && u < nu)
+                                    ? reinterpret_cast<const uint4*>(V + (int64_t)(i0 + t) * ldv)[u] : zero;
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                const int u = b0 + r * bd;
+                if (u >= nu) break;
+                if (have) {
+#pragma unroll
+                    for (int k = 0; k < VW; ++k)
+#pragma unroll
+                        for (int t = 0; t < GB; ++t) zr[r].x[k] = pk_nfma(hp[t], pv[r][t].x[k], zr[r].x[k]);
+                    reinterpret_cast<uint4*>(z)[u] = zr[r].q;
+                }
+                if (norm) {
+#pragma unroll
+                    for (int k = 0; k < VW; ++k) zz = Ar<T>::fma(zr[r].x[k], zr[r].x[k], zz);
+                } else {
+#pragma unroll
+                    for (int t = 0; t < GB; ++t)
+#pragma unroll
+                        for (int k = 0; k < VW; ++k) a[t] = Ar<T>::fma(v[r][t].x[k], zr[r].x[k], a[t]);
+                    if (last) {
+#pragma unroll
+                        for (int k = 0; k < VW; ++k) {
+                            T vj = v[r][0].x[k];
+#pragma unroll
+                            for (int t = 1; t < GB; ++t)
+                                if (t == cnt - 1) vj = v[r][t].x[k];
+#pragma unroll
+                            for (int t = 0; t < GB; ++t) q[t] = Ar<T>::fma(v[r][t].x[k], vj, q[t]);
+                        }
+                    }
+                }
+            }
+        }
+        if (norm) a[0] = zz;
+        warp_multi_sum<GB>(a);
+        if (last) warp_multi_sum<GB>(q);
+        if ((lane & (32 / GB - 1)) == 0) {
+            sh.w[warp_multi_index<GB>(lane)][w] = a[0];
+            sh.w[GB + warp_multi_index<GB>(lane)][w] = last ? q[0] : T(0);
+        }
+        __syncthreads();
+        for (int val = w; val < 2 * GB; val += bd >> 5) {
+            T t = lane < (bd >> 5) ? sh.w[val][lane] : T(0);
+            t = warp_sum(t);
+            if (lane == 0) sh.tot[val] = t;
+        }
+        __syncthreads();
+        if (norm) break;
+        if (w == 0) {
+            T row[GB];
+            group_rows<T, GB>(row, tri + (int64_t)i0 * GB, last ? cnt - 1 : cnt);
+            const T h = group_coeff<T, GB>(row, sh.tot, cnt, last);
+            if (lane < GB) sh.h[lane] = lane < cnt ? h : T(0);
+            if (lane < cnt) hcol[i0 + lane] = (double)h;
+            if (last) group_new_row<T, GB>(row, sh.tot, sh.tri, cnt, tri + (int64_t)j * GB);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < GB; ++t) hp[t] = sh.h[t];
+    }
+    const T hn = Ar<T>::sqrt(sh.tot[0]);
+    const bool nz = hn > T(0) && isfinite((double)hn);
+    T* vn = V + (int64_t)(j + 1) * ldv;
+    if (nz || vn != z) {
+        const Quot<T> by(hn);
+        for (int u = tid; u < nu; u += bd) {
+            Unit x;
+            x.q = reinterpret_cast<const uint4*>(z)[u];
+#pragma unroll
+            for (int k = 0; k < VW; ++k)
+                if (nz) x.x[k] = by(x.x[k]);
+            reinterpret_cast<uint4*>(vn)[u] = x.q;
+        }
+    }
+    return hn;
+}
 
 struct PairState {
     int32_t* status;   // 0 active; 1 nbe <= u; 2 ||d|| <= u ||x||; 3 stagnation; -1 non-finite
@@ -214,7 +350,7 @@ __global__ void __launch_bounds__(512, 1) k_gmres_batch(const __grid_constant__ 
                                                       const int32_t* __restrict__ order, int npairs, int* queue,
                                                       const int32_t* __restrict__ status, const double* __restrict__ R,
                                                       double* __restrict__ X, T* Vws, T* Wws, double* Yws, int64_t ldv,
-                                                      double* Hws, double* Sws, int kmax, double tau, int zcap,
+                                                      double* Hws, double* Sws, T* Tws, int kmax, double tau, int zcap,
                                                       int32_t* __restrict__ iters,
                                                       int32_t* __restrict__ steps, double* __restrict__ relres,
                                                       double* __restrict__ dmax, double* __restrict__ dxmax,
@@ -222,10 +358,20 @@ __global__ void __launch_bounds__(512, 1) k_gmres_batch(const __grid_constant__ 
     extern __shared__ __align__(16) unsigned char s_dyn[];
     T* const s_z = reinterpret_cast<T*>(s_dyn);
     __shared__ T s_w[33];
+    __shared__ StreamShared<T> s_st;
+    __shared__ GivensBatch s_giv;
     __shared__ double s_d[33];
     __shared__ int s_p, s_done;
     __shared__ double s_res;
-    using Ar = BAr<T>;
+    // the matrices' descriptors: read by reference out of line, so from shared memory (a
+    // reference to a kernel parameter makes every thread copy it to its stack)
+    __shared__ BMDev s_A, s_M;
+    if (threadIdx.x == 0) {
+        s_A = Av;
+        s_M = Mv;
+    }
+    __syncthreads();
+    using Ar = bspai::Ar<T>;
     const int tid = threadIdx.x, bd = blockDim.x;
     T* V = Vws + (int64_t)blockIdx.x * ldv * (kmax + 1);
     T* w = Wws + (int64_t)blockIdx.x * ldv;
@@ -233,7 +379,9 @@ __global__ void __launch_bounds__(512, 1) k_gmres_batch(const __grid_constant__ 
     double* cs = Sws + (int64_t)blockIdx.x * 4 * (kmax + 2);
     double* sn = cs + (kmax + 2);
     double* g = sn + (kmax + 2);
-    double* y = g + (kmax + 2);
+    T* tri = Tws + (int64_t)blockIdx.x * 5 * (kmax + 1);
+    T* yt = tri + 4 * (kmax + 1);  // y in u_g
+    double* ys = Yws + (int64_t)blockIdx.x * ldv;
     while (true) {
         if (tid == 0) s_p = atomicAdd(queue, 1);
         __syncthreads();
@@ -247,7 +395,7 @@ __global__ void __launch_bounds__(512, 1) k_gmres_batch(const __grid_constant__ 
         const double* rr = R + (int64_t)rhs * n;
         double* xx = X + (int64_t)rhs * n;
         // s = M r (Alg 2.3), stored in u_g; beta = ||s||_2
-        rows_apply<double, T, MS>(Mv, r0, ns, rr, V, Yws + (int64_t)blockIdx.x * ldv);
+        rows_apply<double, T, MS>(s_M, r0, ns, rr, V, ys);
         T acc = T(0);
         for (int lr = tid; lr < ns; lr += bd) acc = Ar::add(acc, Ar::mul(V[lr], V[lr]));
         const T beta = Ar::sqrt(block_sum(acc, s_w));
@@ -260,62 +408,22 @@ __global__ void __launch_bounds__(512, 1) k_gmres_batch(const __grid_constant__ 
             for (int j = 0; j < kmax; ++j) {
                 __syncthreads();
                 const T* vj = V + (int64_t)j * ldv;
-                rows_apply<T, T, 0>(Av, r0, ns, vj - r0, w, nullptr);
+                if (tid < 32) ask_rows(s_M, r0, ns);  // while A v_j runs
+                rows_apply<T, T, 0>(s_A, r0, ns, vj - r0, w, nullptr);
                 __syncthreads();
                 T* z = ns <= zcap ? s_z : V + (int64_t)(j + 1) * ldv;
-                rows_apply<T, T, MS>(Mv, r0, ns, w - r0, z, Yws + (int64_t)blockIdx.x * ldv);
-                // modified Gram-Schmidt: pass i updates z by the previous coefficient and
-                // dots it with v_i; the last pass forms ||z||_2 (each thread owns its rows of z)
-                T hprev = T(0);
-                for (int i = 0; i <= j + 1; ++i) {
-                    const T* vi = V + (int64_t)(i <= j ? i : j) * ldv;
-                    const T* vp = V + (int64_t)(i > 0 ? i - 1 : 0) * ldv;
-                    T a = T(0);
-                    // U rows of the thread at a time, all their loads issued before
-                    // any store (z shares V's storage, so without this every load
-                    // would wait for the previous row's store); the rows are still
-                    // accumulated in the order tid, tid + bd, tid + 2 bd, ...
-                    for (int b0 = tid; b0 < ns; b0 += bd * U) {
-                        T zr[U], pv[U], iv[U];
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const int lr = b0 + u * bd;
-                            if (lr < ns) {
-                                zr[u] = z[lr];
-                                pv[u] = i > 0 ? vp[lr] : T(0);
-                                iv[u] = i <= j ? vi[lr] : T(0);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const int lr = b0 + u * bd;
-                            if (lr < ns) {
-                                if (i > 0) {
-                                    zr[u] = Ar::sub(zr[u], Ar::mul(hprev, pv[u]));
-                                    z[lr] = zr[u];
-                                }
-                                a = Ar::add(a, Ar::mul(i <= j ? iv[u] : zr[u], zr[u]));
-                            }
-                        }
-                    }
-                    const T h = block_sum(a, s_w);
-                    if (i <= j) {
-                        if (tid == 0) H[(int64_t)j * (kmax + 1) + i] = (double)h;
-                        hprev = h;
-                    } else {
-                        const T hn = Ar::sqrt(h);
-                        // v_{j+1} = z / h_{j+1,j} into the basis (in place when z lives there)
-                        const bool nz = hn > T(0) && isfinite((double)hn);
-                        T* vn = V + (int64_t)(j + 1) * ldv;
-                        if (nz || vn != z)
-                            for (int lr = tid; lr < ns; lr += bd) vn[lr] = nz ? Ar::div(z[lr], hn) : z[lr];
-                        if (tid == 0) {
-                            double rs;
-                            int dn;
-                            givens_pair(j, kmax, (double)hn, H, cs, sn, g, tau, (double)beta, &rs, &dn);
-                            s_res = rs;
-                            s_done = dn;
-                        }
+                rows_apply<T, T, MS>(s_M, r0, ns, w - r0, z, ys);
+                __syncthreads();  // z's rows change hands
+                const T hn = stream_mgs<T, U>(s_st, V, ldv, ns, j, z, H + (int64_t)j * (kmax + 1), tri);
+                if (tid >= bd - 32) ask_rows(s_A, r0, ns);  // the next step's, while the rotations run
+                if (tid < 32) {
+                    __syncwarp();
+                    double rs = 0.0;
+                    int dn = 0;
+                    givens_pair(s_giv, j, kmax, (double)hn, H, cs, sn, g, tau, (double)beta, &rs, &dn);
+                    if (tid == 0) {
+                        s_res = rs;
+                        s_done = dn;
                     }
                 }
                 __syncthreads();
@@ -327,22 +435,33 @@ __global__ void __launch_bounds__(512, 1) k_gmres_batch(const __grid_constant__ 
                 res = s_res;
                 if (s_done) break;
             }
-            // y = R^-1 g, column-oriented back substitution (fp64)
+            // y = R^-1 g, column-oriented back substitution (fp64), by one warp
             __syncthreads();
-            for (int i = k - 1; i >= 0; --i) {
-                const double* hc = H + (int64_t)i * (kmax + 1);
-                if (tid == 0) y[i] = __ddiv_rn(g[i], hc[i]);
-                __syncthreads();
-                const double yi = y[i];
-                for (int t = tid; t < i; t += bd) g[t] = __dsub_rn(g[t], __dmul_rn(hc[t], yi));
-                __syncthreads();
+            if (tid < 32) {
+                for (int i = k - 1; i >= 0; --i) {
+                    const double* hc = H + (int64_t)i * (kmax + 1);
+                    const double yi = __ddiv_rn(g[i], hc[i]);
+                    if (tid == 0) yt[i] = from_f64<T>(yi);
+                    for (int t = tid; t < i; t += 32) g[t] = __dsub_rn(g[t], __dmul_rn(hc[t], yi));
+                    __syncwarp();
+                }
             }
+            __syncthreads();
         }
         // d = V y in u_g, x += d in fp64
         double dm = 0.0, xm = 0.0;
         for (int lr = tid; lr < ns; lr += bd) {
+            // in order of jj, eight columns' loads ahead of their additions
             T a = T(0);
-            for (int jj = 0; jj < k; ++jj) a = Ar::add(a, Ar::mul(V[(int64_t)jj * ldv + lr], from_f64<T>(y[jj])));
+            int jj = 0;
+            for (; jj + 8 <= k; jj += 8) {
+                T v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = V[(int64_t)(jj + u) * ldv + lr];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) a = Ar::add(a, Ar::mul(v[u], yt[jj + u]));
+            }
+            for (; jj < k; ++jj) a = Ar::add(a, Ar::mul(V[(int64_t)jj * ldv + lr], yt[jj]));
             const double d = (double)a;
             const double xn = __dadd_rn(xx[r0 + lr], d);
             xx[r0 + lr] = xn;
@@ -616,6 +735,7 @@ template <int P>
 __global__ void __launch_bounds__(kTeamBD, 1) k_gmres_team(const __grid_constant__ TeamArgs a) {
     constexpr int BD = kTeamBD;
     extern __shared__ float s_y[];  // y of the pair in u_g (kmax entries)
+    __shared__ GivensBatch s_giv;
     __shared__ float s_wf[32];
     __shared__ double s_wd[32];
     __shared__ float s_totf;
@@ -722,12 +842,15 @@ __global__ void __launch_bounds__(kTeamBD, 1) k_gmres_team(const __grid_constant
                 __syncthreads();
                 const float hn = team_mgs<P>(V, ldv, Z, lo, nb, j, kmax, H, ts, s_wf, &s_totf, &s_ok);
                 if (!s_ok) return;
-                if (rank == 0 && tid == 0) {
-                    double rs;
-                    int dn;
-                    givens_pair(j, kmax, (double)hn, H, cs, sn, g, a.tau, (double)beta, &rs, &dn);
-                    s_res = rs;
-                    s_done = dn;
+                if (rank == 0 && tid < 32) {
+                    __syncwarp();
+                    double rs = 0.0;
+                    int dn = 0;
+                    givens_pair(s_giv, j, kmax, (double)hn, H, cs, sn, g, a.tau, (double)beta, &rs, &dn);
+                    if (tid == 0) {
+                        s_res = rs;
+                        s_done = dn;
+                    }
                 }
                 __syncthreads();
                 // every rank learns rank 0's stopping decision (the next barrier is the loop's)
@@ -903,32 +1026,39 @@ static int occupancy_blocks(BatchKernel<T> kern, int bd, size_t smem, int* occ) 
     return BSPAI_OK;
 }
 
-// The largest z_shared_rows for this kernel and CTA size that keeps the CTAs per
-// SM its registers allow (0 when none fit); raises the kernel's dynamic shared
-// memory limit to the opt-in maximum on the way.
+// z_shared_rows of a kernel and CTA size, with the CTAs per SM its registers allow:
+// the most rows a schedule may name (`most`: the SM's shared memory among those CTAs,
+// less 1 KB per CTA that the system reserves and the small static part that has
+// always been set aside) and the most a launch gives (`fit`: what the kernel's own
+// static part leaves; a pair between the two keeps z in memory).  Raises the kernel's
+// dynamic shared memory limit to the opt-in maximum on the way.
 template <typename T>
-static int zcap_limit(BatchKernel<T> kern, int bd, int* zmax) {
+static int zcap_limit(BatchKernel<T> kern, int bd, int* most, int* fit) {
+    constexpr int kStaticPart = sizeof(T) == 4 ? 416 : 552;
     int dev = 0, sm_bytes = 0, blk_bytes = 0, occ0 = 0;
     cudaFuncAttributes fa;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
     CUDA_TRY(cudaDeviceGetAttribute(&blk_bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
-    const int dyn_max = blk_bytes - (int)fa.sharedSizeBytes;
-    CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max));
+    CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  blk_bytes - (int)fa.sharedSizeBytes));
     int rc = occupancy_blocks<T>(kern, bd, 0, &occ0);
     if (rc) return rc;
-    *zmax = 0;
+    *most = *fit = 0;
     if (occ0 < 1) return BSPAI_OK;
-    // 1 KB of shared memory per CTA is reserved by the system
-    int bytes = sm_bytes / occ0 - (int)fa.sharedSizeBytes - 1024;
-    if (bytes > dyn_max) bytes = dyn_max;
-    for (int z = bytes / (int)sizeof(T) / 32 * 32; z >= 32; z -= 256) {
+    auto rows = [&](int part) {
+        int bytes = sm_bytes / occ0 - part - 1024;
+        if (bytes > blk_bytes - part) bytes = blk_bytes - part;
+        return bytes > 0 ? bytes / (int)sizeof(T) / 32 * 32 : 0;
+    };
+    *most = rows(kStaticPart);
+    for (int z = rows((int)fa.sharedSizeBytes); z >= 32; z -= 256) {
         int occ = 0;
         if ((rc = occupancy_blocks<T>(kern, bd, sizeof(T) * (size_t)z, &occ))) return rc;
         if (occ >= occ0) {
-            *zmax = z;
-            return BSPAI_OK;
+            *fit = z;
+            break;
         }
     }
     return BSPAI_OK;
@@ -1040,18 +1170,37 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
     }
     const BMDev Av = single_bucket_view(A->sell, u_p == BSPAI_FP64 ? (const void*)A->val64 : (const void*)A->val32,
                                         u_p);
-    const BMDev Mv = BM->dev();
+    const BMDev Mv = compact_buckets(BM->dev());  // empty buckets add nothing
     // schedule: forced by the caller's thread, cached per batch shape, or tuned below
     const size_t ws_budget = (size_t)24 << 30;
     const int sms = num_sms();
     const int nmax32 = (int)ceil_div(nmax > 0 ? nmax : 1, 32) * 32;
+    // the z-in-shared-memory limits of each (tile, bucket schedule, CTA size), whose query
+    // also raises the kernels' dynamic shared memory limit before any launch
+    const int cand_bd[3] = {128, 256, 512};
+    int zmost[2][2][3], zgive[2][2][3];  // rows of z a schedule may name, and a launch gives
+    for (int u = 0; u < 2; ++u)
+        for (int m = 0; m < 2; ++m)
+            for (int c = 0; c < 3; ++c)
+                if ((rc = zcap_limit<T>(batch_kernel<T>(u ? MgsU<T>::hi : MgsU<T>::lo, m), cand_bd[c],
+                                        &zmost[u][m][c], &zgive[u][m][c])))
+                    return done(rc);
+    auto zlim = [&](const Sched& c, const int (&t)[2][2][3]) {
+        return t[c.urows == MgsU<T>::hi ? 1 : 0][c.msched ? 1 : 0][c.bd == 512 ? 2 : c.bd == 256 ? 1 : 0];
+    };
+    auto zfit = [&](const Sched& c) { return zlim(c, zmost); };
+    auto launch_z = [&](const Sched& c) {
+        const int z = zlim(c, zgive);
+        return c.zcap < z ? c.zcap : z;
+    };
     auto grid_for = [&](const Sched& c, int* grid) -> int {
         int occ = 0;
-        int r2 = occupancy_blocks<T>(batch_kernel<T>(c.urows, c.msched), c.bd, sizeof(T) * (size_t)c.zcap, &occ);
+        int r2 = occupancy_blocks<T>(batch_kernel<T>(c.urows, c.msched), c.bd, sizeof(T) * (size_t)launch_z(c), &occ);
         if (r2) return r2;
         if (occ < 1) return set_error(BSPAI_ERR_CUDA, "batched GMRES kernel does not fit on an SM");
         const size_t per = sizeof(T) * (size_t)ldv * (kmax + 2) + sizeof(double) * (size_t)ldv +
-                           sizeof(double) * ((size_t)(kmax + 1) * kmax + 4 * (kmax + 2));
+                           sizeof(double) * ((size_t)(kmax + 1) * kmax + 4 * (kmax + 2)) +
+                           sizeof(T) * 5 * (size_t)(kmax + 1);
         int gmax = (int)(ws_budget / per);
         int gr = sms * occ;
         if (o.max_blocks > 0 && gr > o.max_blocks) gr = o.max_blocks;
@@ -1059,22 +1208,6 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
         if (gr > npairs) gr = npairs;
         *grid = gr < 1 ? 1 : gr;
         return BSPAI_OK;
-    };
-    // the z-in-shared-memory limit of each (tile, CTA size), which also raises the
-    // kernels' dynamic shared memory limit before any launch
-    const int cand_bd[3] = {128, 256, 512};
-    int zlim[2][2][3];  // [tile][bucket schedule][CTA size]: rows of z that fit
-    for (int u = 0; u < 2; ++u)
-        for (int m = 0; m < 2; ++m)
-            for (int c = 0; c < 3; ++c)
-                if ((rc = zcap_limit<T>(batch_kernel<T>(u ? MgsU<T>::hi : MgsU<T>::lo, m), cand_bd[c],
-                                        &zlim[u][m][c])))
-                    return done(rc);
-    auto zfit = [&](const Sched& c) {
-        const int u = c.urows == MgsU<T>::hi ? 1 : 0;
-        for (int k = 0; k < 3; ++k)
-            if (cand_bd[k] == c.bd) return zlim[u][c.msched ? 1 : 0][k];
-        return 0;
     };
     // the candidate the tuner tries: every pair of the batch, if it fits
     auto zlimit = [&](const Sched& c) {
@@ -1119,7 +1252,7 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
                     cs.bd = cand_bd[c];
                     cs.urows = u ? MgsU<T>::hi : MgsU<T>::lo;
                     cs.msched = m;
-                    cs.zcap = zs ? (zlim[u][m][c] < nmax32 ? zlim[u][m][c] : nmax32) : 0;
+                    cs.zcap = zs ? (zmost[u][m][c] < nmax32 ? zmost[u][m][c] : nmax32) : 0;
                     int gr;
                     if ((rc = grid_for(cs, &gr))) return done(rc);
                     gmax_all = gr > gmax_all ? gr : gmax_all;
@@ -1136,13 +1269,15 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
     if ((rc = take((void**)&Yws, sizeof(double) * (size_t)gmax_all * ldv))) return done(rc);
     if ((rc = take((void**)&Hws, sizeof(double) * (size_t)gmax_all * (kmax + 1) * kmax))) return done(rc);
     if ((rc = take((void**)&Sws, sizeof(double) * (size_t)gmax_all * 4 * (kmax + 2)))) return done(rc);
+    T* Tws = nullptr;  // the groups' triangles (mgs.cuh), and y in u_g
+    if ((rc = take((void**)&Tws, sizeof(T) * (size_t)gmax_all * 5 * (kmax + 1)))) return done(rc);
     unsigned long long* d_work = nullptr;  // algorithmic work counters of the GMRES launches
     if ((rc = take((void**)&d_work, 2 * sizeof(unsigned long long)))) return done(rc);
     auto launch_gmres = [&](const Sched& c, int grid, const double* Rin, double* Xout, int kcap, double tcap,
                             PairState& St, cudaStream_t st, int np) {
-        batch_kernel<T>(c.urows, c.msched)<<<grid, c.bd, sizeof(T) * (size_t)c.zcap, st>>>(
+        batch_kernel<T>(c.urows, c.msched)<<<grid, c.bd, sizeof(T) * (size_t)launch_z(c), st>>>(
             Av, Mv, row_off, nsys, n, d_order, np, d_queue, St.status, Rin, Xout, Vws, Wws, Yws, ldv, Hws, Sws,
-            kcap, tcap, c.zcap, St.iters, St.steps, St.relres, St.dmax, St.dxmax, d_work);
+            Tws, kcap, tcap, launch_z(c), St.iters, St.steps, St.relres, St.dmax, St.dxmax, d_work);
         note_launch();
         return cudaGetLastError();
     };

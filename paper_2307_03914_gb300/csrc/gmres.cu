@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_mgs(T* __restri
     __shared__ int s_j, s_done, s_kmax;
     __shared__ unsigned s_seq;
     __shared__ T s_w[2 * GB][32], s_tot[2 * GB], s_h[GB], s_tri[GB][GB];
+    __shared__ GivensBatch s_giv;
     if (threadIdx.x == 0) {
         s_j = st->j;
         s_done = st->done;
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_mgs(T* __restri
             st->bar.seq = tag;
         }
         __syncwarp();
-        if (!givens_column<T>(j, kmax, H, cs, sn, g, st, hq, tag, tmo) && lane == 0) {
+        if (!givens_column<T>(s_giv, j, kmax, H, cs, sn, g, st, hq, tag, tmo) && lane == 0) {
             st->status = BSPAI_TIMEOUT;
             st->done = 1;
         }
@@ -265,6 +266,7 @@ __device__ __forceinline__ void mgs_kernel(typename I::type* __restrict__ V, int
     typedef typename I::type T;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ MgsShared<I> sh;
+    __shared__ GivensBatch s_giv;
     __shared__ unsigned s_seq;
     __shared__ int s_j, s_done, s_kmax;
     const int tid = threadIdx.x;
@@ -302,7 +304,7 @@ __device__ __forceinline__ void mgs_kernel(typename I::type* __restrict__ V, int
                 unit_load<I>(R, zg, u, z + u * I::PN);
             }
         }
-        const MgsIo io{tags, hq, tri, &st->bar, tmo, G, bulk, blockIdx.x == 0, blockIdx.x == 0};
+        const MgsIo io{tags, hq, tri, &st->bar, tmo, G, bulk, blockIdx.x == 0, blockIdx.x == 0, nullptr};
         unsigned seq = seq0, phase = 0;
         T hz;
         if (!mgs_passes<I>(sh, io, R, z, smraw, zs, V + r0, ldv, j, tag, seq, phase, hz)) {
@@ -330,7 +332,7 @@ __device__ __forceinline__ void mgs_kernel(typename I::type* __restrict__ V, int
         }
     }
     if (rotates && tid < 32) {
-        const bool ok = givens_column<T>(j, kmax, H, cs, sn, g, st, hq, tag, tmo);
+        const bool ok = givens_column<T>(s_giv, j, kmax, H, cs, sn, g, st, hq, tag, tmo);
         if (tid == 0) {
             if (ok) {
                 // every block has read seq0 (the reductions are complete): advance it

@@ -229,6 +229,7 @@ struct MgsIo {
     int bulk;     // poll by bulk copies (instances that have them compiled in)
     bool tri_out; // this block writes new rows of tri
     bool hq_out;  // this block publishes the coefficients
+    double* hcol; // or (not null) writes them here: the column of H itself
 };
 
 template <typename T, int VW_, int NU_, int BD_, int GB_, int S_, bool BULK_, bool ZS_>
@@ -276,6 +277,16 @@ __device__ __forceinline__ void mgs_shared_init(MgsShared<I>& sh) {  // one thre
         for (int w = 0; w < I::NPW; ++w) mbar_init(&sh.mbar[w], 1);
     }
     mbar_init_fence();
+}
+// before a further mgs_shared_init on the same storage (one thread, every copy complete)
+template <class I>
+__device__ __forceinline__ void mgs_shared_retire(MgsShared<I>& sh) {
+#pragma unroll
+    for (int s = 0; s < I::S; ++s) mbar_inval(&sh.full[s]);
+    if constexpr (I::BULK) {
+#pragma unroll
+        for (int w = 0; w < I::NPW; ++w) mbar_inval(&sh.mbar[w]);
+    }
 }
 
 template <class I>
@@ -565,8 +576,10 @@ __device__ __forceinline__ bool mgs_passes(MgsShared<I>& sh, const MgsIo& io, co
         if (w == 0) {
             const T h = group_coeff<T, GB>(rowt, sh.tot, cnt, last);
             if (lane < GB) sh.h[lane] = lane < cnt ? h : T(0);
-            if (io.hq_out && lane < cnt)
-                tag_publish(h, io.hq + (int64_t)(i0 + lane) * TagWords<T>::W, hq_tag);
+            if (lane < cnt) {
+                if (io.hcol) io.hcol[i0 + lane] = (double)h;
+                else if (io.hq_out) tag_publish(h, io.hq + (int64_t)(i0 + lane) * TagWords<T>::W, hq_tag);
+            }
         }
         __syncthreads();
         if (!*(volatile int*)&sh.ok) {
@@ -601,7 +614,7 @@ __device__ __forceinline__ bool mgs_passes(MgsShared<I>& sh, const MgsIo& io, co
         ++seq;
         mgs_arrive<I>(sh, io, seq, w == 0);
         mgs_poll<I>(sh, io, seq, w == 0, phase);
-        if (w == 0 && lane == 0 && io.hq_out)
+        if (w == 0 && lane == 0 && io.hq_out && !io.hcol)
             tag_publish(Ar<T>::sqrt(sh.tot[0]), io.hq + (int64_t)(j + 1) * TagWords<T>::W, hq_tag);
         __syncthreads();
     }
@@ -641,17 +654,44 @@ __device__ __forceinline__ void givens_finish(int j, int kmax, double hn, double
     st->done = (res <= lvl) || hn == 0.0 || k >= kmax || !fin;
 }
 
+// The earlier rotations applied by one warp to up to 32 entries of a column (lane t:
+// entry h of the column and the rotation c, s that takes it in), carry the entry
+// handed on from the ones before.  Only the carry is a chain, -s carry + c h, two
+// dependent operations of 64 cycles each on GB300's narrow fp64 pipe; the products
+// c h and the rotated entries c carry + s h are formed 32 at a time around it (per
+// rotation 175 cycles, against 364 with both rows of a rotation inside the chain).
+struct GivensBatch {
+    double s[32], m[32];
+};
+// entries [from, to) of the batch, whose lanes hold c, s, h; lane t keeps the carry its rotation met
+__device__ __forceinline__ void givens_chain(GivensBatch& gb, int from, int to, double c, double s, double h,
+                                             double& carry, double& met) {
+    const int lane = threadIdx.x & 31;
+    if (lane >= from && lane < to) {
+        gb.s[lane] = -s;
+        gb.m[lane] = __dmul_rn(c, h);
+    }
+    __syncwarp();
+#pragma unroll 4
+    for (int t = from; t < to; ++t) {
+        const double ms = gb.s[t], m = gb.m[t];
+        if (lane == t) met = carry;
+        carry = __dadd_rn(__dmul_rn(ms, carry), m);
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ double givens_entry(double c, double s, double h, double met) {
+    return __dadd_rn(__dmul_rn(c, met), __dmul_rn(s, h));
+}
+
 // The earlier rotations applied to column j of H by one warp, entry by entry as
 // the coefficients arrive in hq (tag: this step's; the words are not overwritten
 // within a step, so a warp that starts late misses nothing), then the new
-// rotation, g and the tau test.  One rotation depends on the one before, on
-// GB300's narrow fp64 pipe: the two rows of a rotation run in neighbouring lanes
-// (two multiplies and one addition issued per rotation instead of four and two)
-// and the stored rotations are read 32 at a time, ahead of their use.  False
-// after a timeout.
+// rotation, g and the tau test.  False after a timeout.
 template <typename T>
-__device__ bool givens_column(int j, int kmax, double* __restrict__ H, double* cs, double* sn, double* g,
-                              GmresState* st, const unsigned long long* hq, unsigned tag, unsigned long long tmo) {
+__device__ bool givens_column(GivensBatch& gb, int j, int kmax, double* __restrict__ H, double* cs, double* sn,
+                              double* g, GmresState* st, const unsigned long long* hq, unsigned tag,
+                              unsigned long long tmo) {
     constexpr unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     double* __restrict__ hc = H + (int64_t)j * (kmax + 1);
@@ -665,6 +705,7 @@ __device__ bool givens_column(int j, int kmax, double* __restrict__ H, double* c
         T hv = T(0);
         bool have = lane >= nin;
         int taken = 0;
+        double met = 0.0;
         unsigned long long t0 = 0;
         for (int it = 0; taken < nin; ++it) {
             if (!have) have = tag_read(hq + (int64_t)i * TagWords<T>::W, tag, &hv);
@@ -687,24 +728,19 @@ __device__ bool givens_column(int j, int kmax, double* __restrict__ H, double* c
             }
             t0 = 0;
             const double hd = (double)hv;
-            for (; taken < upto && taken < nin; ++taken) {
-                const double h = __shfl_sync(full, hd, taken);
-                const int e = base + taken;
-                if (e == j + 1) {
-                    hn = h;
-                } else if (e == 0) {
-                    carry = h;
-                } else {
-                    const double c = __shfl_sync(full, ci, taken), s = __shfl_sync(full, si, taken);
-                    // even lanes: c carry + s h (the rotated entry e - 1); odd lanes: -s carry + c h
-                    const bool odd = lane & 1;
-                    const double m2 = __dmul_rn(odd ? c : s, h);
-                    const double r = __dadd_rn(__dmul_rn(odd ? -s : c, carry), m2);
-                    if (lane == 0) hc[e - 1] = r;
-                    carry = __shfl_sync(full, r, 1);
-                }
+            int to = upto;
+            if (base + to == j + 2) {  // the last word is h_{j+1,j}
+                --to;
+                hn = __shfl_sync(full, hd, to);
             }
+            if (base == 0 && taken == 0) {
+                carry = __shfl_sync(full, hd, 0);
+                taken = 1;
+            }
+            givens_chain(gb, taken, to, ci, si, hd, carry, met);
+            taken = upto;
         }
+        if (rot) hc[i - 1] = givens_entry(ci, si, (double)hv, met);
     }
     if (lane == 0) givens_finish(j, kmax, hn, carry, hc, cs, sn, g, st);
     return true;
