@@ -6,7 +6,8 @@
 // with D = diag(1 / max_i |a_ji|), and the left preconditioner is M = M'^T D,
 // so column k of M' is row k of M and column j of B is row j of A times d_j.
 //
-// One warp per column k, in u_f = fp32:
+// In u_f = fp32 a team of threads per column holds the block in registers
+// (spai_team.cuh).  The larger blocks, and u_f = fp16, take one warp per column k:
 //   J_k   = pattern of row k of M (ascending)
 //   I_k   = shadow: the union of the columns of rows J_k of A, sorted (bitonic
 //           sort of the gathered candidates in shared memory, then a
@@ -18,8 +19,11 @@
 //   sbar  = Abar mbar - ebar recomputed from the gathered rows; ||sbar||_2
 // and M[k, J_k[q]] = mbar_q d_{J_k[q]} is written into the SELL slots of row k.
 #include <climits>
+#include <type_traits>
+#include <utility>
 
 #include "common.cuh"
+#include "spai_team.cuh"
 
 namespace bspai {
 
@@ -70,13 +74,6 @@ __global__ void __launch_bounds__(256) k_spai_sizes(int n, const int64_t* __rest
     }
 }
 
-struct SpaiCounters {
-    int n_conv;
-    int n_rankdef;
-    float max_resid;
-    int n_nonfinite;  // entries of M outside the range of u_f (fp16: |m| >= 65520 rounds to Inf)
-};
-
 // Shared memory of one warp (bytes): dJ (fp64, |J|), J, mbar, R's diagonal,
 // A's row start and the entry offset of every j in J (int32, |J| + 1), the
 // sort buffer (lp2), I, Abar (|I| x |J|), ebar / Q^T ebar, sbar, and per
@@ -107,13 +104,19 @@ __global__ void __launch_bounds__(256, 5) k_spai(int n, const int32_t* __restric
                                                const int64_t* __restrict__ msptr, const int32_t* __restrict__ mcol,
                                                const int32_t* __restrict__ mrowlen, float* __restrict__ mval,
                                                float* __restrict__ resid, float spai_eps, float u_f, int jmax,
-                                               int lmax, int lp2, SpaiCounters* __restrict__ cnt) {
+                                               int lmax, int lp2, SpaiCounters* __restrict__ cnt,
+                                               const int* __restrict__ list) {
     using F = UfOps<H>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    const int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-    if (k >= n) return;
+    int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
+    if (list) {  // the columns k_spai_team left (n: how many the launch covers)
+        if (k >= cnt->n_left) return;
+        k = list[k];
+    } else if (k >= n) {
+        return;
+    }
 
     // per-warp shared-memory carve-up
     const size_t per_warp = spai_warp_bytes(jmax, lmax, lp2);
@@ -382,6 +385,24 @@ __global__ void __launch_bounds__(256, 5) k_spai(int n, const int32_t* __restric
     }
 }
 
+// The team instances, smallest first
+struct SpaiTeamKernel {
+    void (*fn)(int, const int32_t*, const int32_t*, const double*, const double*, const int64_t*, const int32_t*,
+               const int32_t*, float*, float*, float, float, SpaiCounters*, int*);
+    int cols, slots, rows, per_block, threads;
+    size_t smem;
+};
+template <int TS, int E, int NR, int NC, int BD, int MINB>
+constexpr SpaiTeamKernel spai_team() {
+    typedef SpaiShape<TS, E, NR, NC, BD> Sh;
+    return {k_spai_team<TS, E, NR, NC, BD, MINB>, NC, Sh::SLOTS, Sh::ROWS, Sh::COLS, BD, Sh::smem};
+}
+static const SpaiTeamKernel kSpaiTeams[] = {
+    spai_team<8, 8, 4, 8, 256, 3>(),    // 5- and 7-point stencils: |J| <= 8, 64 candidates, 32 rows
+    spai_team<8, 16, 4, 12, 256, 2>(),  // 9-point: |J| <= 12, 128 candidates, 32 rows
+    spai_team<128, 4, 4, 24, 128, 4>(), // |J| <= 24, 512 candidates and rows
+};
+
 // fp64 values rounded once to fp16 (held in fp64), for an M imported in u_f = fp16
 __global__ void k_round_f16_of_f64(int64_t n, const double* __restrict__ x, double* __restrict__ y) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -433,11 +454,13 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
     double* d = nullptr;
     int* sizes = nullptr;
     SpaiCounters* cnt = nullptr;
+    int* left = nullptr;  // columns that k_spai_team left to k_spai
     int st_ = BSPAI_OK;
     auto fail = [&](int code) {
         dfree(d, s);
         dfree(sizes, s);
         dfree(cnt, s);
+        dfree(left, s);
         bspai_free(M);
         return code;
     };
@@ -487,16 +510,50 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
     if (n > 0) {
         ProfScope ps(BSPAI_K_SPAI, s);
         const bool h = u_f == BSPAI_FP16;
-        e = cudaFuncSetAttribute(h ? k_spai<true> : k_spai<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
+        const float uf = h ? 4.8828125e-04f : 5.9604644775390625e-08f;  // 2^-11 or 2^-24, the rank test's unit roundoff
+        auto attr = [&](const void* fn, size_t bytes) {
+            return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        };
+        e = attr(h ? (const void*)k_spai<true> : (const void*)k_spai<false>, smem);
         if (e != cudaSuccess) return fail(cuda_error(e, "spai smem attribute", __FILE__, __LINE__));
-        // u_f: 2^-24 (fp32) or 2^-11 (fp16), the rank test's unit roundoff
-        (h ? k_spai<true> : k_spai<false>)<<<(unsigned)ceil_div(n, warps), 32 * warps, smem, s>>>(
-            n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
-            (float)spai_eps, h ? 4.8828125e-04f : 5.9604644775390625e-08f, jmax, lmax, lp2, cnt);
-        note_launch();
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(cuda_error(e, "k_spai", __FILE__, __LINE__));
+        // fp32: the smallest team whose columns and candidates hold every block (its rows are
+        // checked per column); half, and larger blocks, a warp per column
+        const SpaiTeamKernel* tk = nullptr;
+        if (!h)
+            for (const SpaiTeamKernel& c : kSpaiTeams)
+                if (!tk && jmax <= c.cols && lmax <= c.slots) tk = &c;
+        if (tk) {
+            if ((st_ = dalloc_t(&left, (size_t)n, s))) return fail(st_);
+            e = attr((const void*)tk->fn, tk->smem);
+            if (e != cudaSuccess) return fail(cuda_error(e, "spai team smem attribute", __FILE__, __LINE__));
+            tk->fn<<<(unsigned)ceil_div(n, tk->per_block), tk->threads, tk->smem, s>>>(
+                n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
+                (float)spai_eps, uf, cnt, left);
+            note_launch();
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return fail(cuda_error(e, "k_spai_team", __FILE__, __LINE__));
+            if (lmax > tk->rows) {  // a shadow could be larger than the team's rows
+                int nl = 0;
+                e = cudaMemcpyAsync(&nl, &cnt->n_left, sizeof nl, cudaMemcpyDeviceToHost, s);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+                if (e != cudaSuccess) return fail(cuda_error(e, "spai columns left", __FILE__, __LINE__));
+                if (nl > 0) {
+                    k_spai<false><<<(unsigned)ceil_div(nl, warps), 32 * warps, smem, s>>>(
+                        nl, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
+                        (float)spai_eps, uf, jmax, lmax, lp2, cnt, left);
+                    note_launch();
+                    e = cudaGetLastError();
+                    if (e != cudaSuccess) return fail(cuda_error(e, "k_spai", __FILE__, __LINE__));
+                }
+            }
+        } else {
+            (h ? k_spai<true> : k_spai<false>)<<<(unsigned)ceil_div(n, warps), 32 * warps, smem, s>>>(
+                n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
+                (float)spai_eps, uf, jmax, lmax, lp2, cnt, nullptr);
+            note_launch();
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return fail(cuda_error(e, "k_spai", __FILE__, __LINE__));
+        }
     }
     SpaiCounters hc{};
     e = cudaMemcpyAsync(&hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, s);
@@ -505,6 +562,7 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
     dfree(d, s);
     dfree(sizes, s);
     dfree(cnt, s);
+    dfree(left, s);
     if (info) {
         info->n = n;
         info->max_cols = hs[0];
