@@ -242,11 +242,22 @@ int launch_row_abs_sum_max(const Sell& S, const double* val, double* out, cudaSt
 }
 
 // ------------------------------------------------ error-free transformations
-// Knuth TwoSum.
+// s + e = a + b exactly (s = fl(a + b)): Dekker's FastTwoSum, three operations
+// where Knuth's TwoSum takes six, on the operands ordered by exponent.  The order
+// comes from their high words (integer work: GB300's fp64 pipe is what bounds the
+// residual); an exponent not below the other's is all FastTwoSum asks for, so e is
+// the same exact error, bit for bit.
 __device__ __forceinline__ void dd_two_sum(double a, double b, double& s, double& e) {
+    const bool sw = (__double2hiint(a) & 0x7fffffff) < (__double2hiint(b) & 0x7fffffff);
+    const double big = sw ? b : a, small = sw ? a : b;
     s = __dadd_rn(a, b);
-    double bv = __dsub_rn(s, a);
-    e = __dadd_rn(__dsub_rn(a, __dsub_rn(s, bv)), __dsub_rn(b, bv));
+    e = __dsub_rn(small, __dsub_rn(s, big));
+}
+// |v| as an ordered integer for maxima (NaN: Inf, or nothing for `skip`), and back
+__device__ __forceinline__ unsigned long long abs_bits(double v, bool skip = false) {
+    const unsigned long long inf = 0x7ff0000000000000ull;
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return u <= inf ? u : skip ? 0ull : inf;
 }
 // One term of the compensated dot product Dot2 (Ogita, Rump and Oishi, 2005):
 // the running sum p absorbs -ph by TwoSum, the running error s collects the
@@ -261,7 +272,10 @@ __device__ __forceinline__ void dot2_sub(double& p, double& s, double ph, double
 // r = b - A x, each product split exactly by an FMA and the terms summed by
 // Dot2 in ascending column order (DD = true: u_r ~ u^2; DD = false is the
 // plain fp64 recurrence), stored in the working precision (U32: rounded to
-// fp32); also max|r| (of the stored r) and max|x| over rows.
+// fp32); also max|r| (of the stored r) and max|x| over rows.  Bound by the fp64
+// pipe: seven operations per entry (170 us at 128^3 at the measured 625 G/s; with
+// TwoSum and fp64 maxima, ten per entry and five per row, it took 311 us; now 236,
+// 241 with one slot's loads at a time).
 template <bool DD, bool U32>
 __global__ void __launch_bounds__(256) k_residual_dd(int n, const int64_t* __restrict__ sptr,
                                                      const int32_t* __restrict__ col,
@@ -269,38 +283,49 @@ __global__ void __launch_bounds__(256) k_residual_dd(int n, const int64_t* __res
                                                      const double* __restrict__ x,
                                                      const double* __restrict__ b, double* __restrict__ r,
                                                      double* __restrict__ norms) {
-    double rabs = 0.0, xabs = 0.0;
+    unsigned long long rabs = 0, xabs = 0;  // maxima as integers: none of the fp64 pipe's time
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t s = i >> 5;
         double hi = b[i], lo = 0.0;
         const int64_t end = sptr[s + 1];
-        for (int64_t p = sptr[s] + (i & 31); p < end; p += kSlice) {
-            const int c = __ldg(col + p);
-            if (c < 0) break;
-            const double a = __ldg(val + p);
-            const double xv = __ldg(x + c);
-            const double ph = __dmul_rn(a, xv);
-            if (DD) {
-                const double pl = __fma_rn(a, xv, -ph);
-                dot2_sub(hi, lo, ph, pl);
-            } else {
-                hi = __dsub_rn(hi, ph);
+        // four slots' columns, then their values and entries of x, ahead of the arithmetic
+        for (int64_t p = sptr[s] + (i & 31); p < end; p += 4 * kSlice) {
+            int c[4];
+            double a[4], xv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c[u] = p + u * kSlice < end ? __ldg(col + p + u * kSlice) : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c[u] >= 0) {
+                    a[u] = __ldg(val + p + u * kSlice);
+                    xv[u] = __ldg(x + c[u]);
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (c[u] < 0) break;
+                const double ph = __dmul_rn(a[u], xv[u]);
+                if (DD) {
+                    const double pl = __fma_rn(a[u], xv[u], -ph);
+                    dot2_sub(hi, lo, ph, pl);
+                } else {
+                    hi = __dsub_rn(hi, ph);
+                }
             }
         }
         double ri = __dadd_rn(hi, lo);
         if (U32) ri = (double)__double2float_rn(ri);
         r[i] = ri;
-        double ra = fabs(ri);
-        if (!(ra <= 1.7976931348623157e308)) ra = __longlong_as_double(0x7ff0000000000000LL);  // NaN -> Inf
-        rabs = fmax(rabs, ra);
-        xabs = fmax(xabs, fabs(x[i]));
+        rabs = max(rabs, abs_bits(ri));
+        xabs = max(xabs, abs_bits(x[i], true));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        rabs = fmax(rabs, __shfl_xor_sync(0xffffffffu, rabs, o));
-        xabs = fmax(xabs, __shfl_xor_sync(0xffffffffu, xabs, o));
+        rabs = max(rabs, __shfl_xor_sync(0xffffffffu, rabs, o));
+        xabs = max(xabs, __shfl_xor_sync(0xffffffffu, xabs, o));
     }
-    if (norms) block_atomic_max_nonneg2(norms, rabs, norms + 1, xabs);
+    if (norms)
+        block_atomic_max_nonneg2(norms, __longlong_as_double((long long)rabs), norms + 1,
+                                 __longlong_as_double((long long)xabs));
 }
 
 // The same residual for nrhs right-hand sides of a block-diagonal batch
@@ -333,17 +358,16 @@ __global__ void __launch_bounds__(256) k_residual_batch(int n, int nrhs, const i
     }
     const double ri = __dadd_rn(hi, lo);
     R[t] = ri;
-    double rabs = fabs(ri), xabs = fabs(x[i]);
-    if (!(rabs <= 1.7976931348623157e308)) rabs = __longlong_as_double(0x7ff0000000000000LL);
+    unsigned long long rabs = abs_bits(ri), xabs = abs_bits(x[i], true);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        rabs = fmax(rabs, __shfl_xor_sync(0xffffffffu, rabs, o));
-        xabs = fmax(xabs, __shfl_xor_sync(0xffffffffu, xabs, o));
+        rabs = max(rabs, __shfl_xor_sync(0xffffffffu, rabs, o));
+        xabs = max(xabs, __shfl_xor_sync(0xffffffffu, xabs, o));
     }
     if ((threadIdx.x & 31) == 0) {
         const int64_t pair = rhs * nsys + slice_seg[s];
-        atomic_max_nonneg(prmax + pair, rabs);
-        atomic_max_nonneg(pxmax + pair, xabs);
+        atomic_max_nonneg(prmax + pair, __longlong_as_double((long long)rabs));
+        atomic_max_nonneg(pxmax + pair, __longlong_as_double((long long)xabs));
     }
 }
 
