@@ -381,7 +381,11 @@ int bspai_gmres(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_t u_g, b
  * the grid reductions' slots by bulk copies into shared memory instead of by
  * loads (at least 16 KB of each basis vector per block and at least 64
  * blocks), 0 otherwise.  Every kernel takes the basis in groups of 1 to 8
- * vectors, one reduction per group.  A query only: nothing is launched or allocated.  n < 1:
+ * vectors, one reduction per group.  (A system of at most 32,768 rows that
+ * max_blocks leaves room for, whose A and M have short rows, takes all its
+ * steps in one launch instead, with the same Gram-Schmidt in groups of 8 on
+ * blocks of 512 threads and its own row products in every SpMV form; the
+ * order alone does not tell, so the query does not.)  A query only: nothing is launched or allocated.  n < 1:
  * BSPAI_ERR_INVALID; another u_g: BSPAI_ERR_UNSUPPORTED. */
 typedef struct {
     int32_t kernel;

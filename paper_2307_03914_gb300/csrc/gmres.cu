@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "mgs.cuh"
+#include "spmv_row.cuh"
 #include "tags.cuh"
 
 namespace bspai {
@@ -305,9 +306,9 @@ __device__ __forceinline__ void mgs_kernel(typename I::type* __restrict__ V, int
             }
         }
         const MgsIo io{tags, hq, tri, &st->bar, tmo, G, bulk, blockIdx.x == 0, blockIdx.x == 0, nullptr};
-        unsigned seq = seq0, phase = 0;
+        unsigned seq = seq0, phase = 0, par = 0;
         T hz;
-        if (!mgs_passes<I>(sh, io, R, z, smraw, zs, V + r0, ldv, j, tag, seq, phase, hz)) {
+        if (!mgs_passes<I>(sh, io, R, z, smraw, zs, V + r0, ldv, j, tag, seq, phase, par, hz)) {
             if (blockIdx.x == 0 && tid == 0) {
                 st->status = BSPAI_TIMEOUT;
                 st->done = 1;
@@ -387,6 +388,281 @@ __global__ void __launch_bounds__(BD, 1) k_mgs_res2(float* __restrict__ V, int64
                                                     unsigned long long* tags, unsigned long long* hq, void* tri,
                                                     unsigned long long tmo, int giv, int bulk) {
     mgs_kernel<ResInst2<P, BD>>(V, ldv, n, st, H, cs, sn, g, tags, hq, tri, tmo, giv, bulk);
+}
+
+// ------------------------------------------------------------------ one launch per run
+// The whole Arnoldi loop of a small system with short rows in one cooperative launch:
+// A v_j, M w and the Gram-Schmidt step of mgs.cuh with z never leaving its registers
+// (fp32: two adjacent rows per thread, fp64: one).  What bounds a small system is
+// latency: with three launches per step, each of a few microseconds of launch, first
+// loads and drain, a step cost 35 us at n = 1,024; here it is two grid exchanges (v_j
+// and w complete) and the reductions.  The row blocks exchange by tagged words;
+// vectors another block writes are read from L2, after release / acquire fences around
+// the exchange.  The last block applies the Givens rotations and decides the stop; the
+// row blocks learn of step j - 1's decision at the end of step j, so at most one step
+// is run in vain, and its column's words (two sets, by the step's parity) are not
+// overwritten before they are read.
+//
+// A row's entries -- columns and values as the product uses them -- are kept in shared
+// memory for the run (at most kCoopRow per row of each matrix, in one fp64 bucket or
+// one or two narrow ones), so that a product waits for one load, x's, instead of a
+// chain of three.  (A launch whose matrices have longer rows stays with the products'
+// own kernels: at 17 and 24 entries per row they took 32 us a step against 57 here.)
+constexpr int kCoopBD = 512;
+constexpr int kCoopRow = 9;
+constexpr int kCoopMax = 32;  // row blocks at most (fp64: twice as many)
+constexpr int kCoopToken = kMgsMaxVals - 1;  // the slots' row of the exchanges without a value
+template <typename T>
+struct CoopInst : MgsInst<T, sizeof(T) == 4 ? 2 : 1, 1, kCoopBD, 8, 8, false, false> {};
+// bytes of a matrix's cached entries: 4 of column and 4 or 8 of value
+template <typename T>
+constexpr size_t coop_cache_bytes(bool wide) {
+    return (size_t)kCoopRow * kCoopBD * CoopInst<T>::VW * (wide ? 12 : 8);
+}
+template <typename T>
+constexpr size_t coop_smem() {  // A's values are T, M's may be fp64 in either case
+    return CoopInst<T>::smem + coop_cache_bytes<T>(sizeof(T) == 8) + coop_cache_bytes<T>(true);
+}
+
+// every row block's writes before it are visible to every row block's L2 reads after it
+template <class I>
+__device__ __forceinline__ void coop_exchange(MgsShared<I>& sh, const MgsIo& io, unsigned seq) {
+    typedef typename I::type T;
+    __syncthreads();
+    if (io.G == 1) return;
+    if (threadIdx.x < 32) {
+        unsigned long long* row =
+            io.tags + (int64_t)((int)(seq & 1u) * kMgsMaxVals + kCoopToken) * kTagMaxBlocks * TagWords<T>::W;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            tag_publish(T(0), row + (int64_t)blockIdx.x * TagWords<T>::W, seq);
+        }
+        T t;
+        if (!tag_poll_row<T>(row, seq, io.G, io.bar, io.tmo, &t) && threadIdx.x == 0) *(volatile int*)&sh.ok = 0;
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+// A matrix's rows of this block in shared memory.  mode: 0 not kept, 1 one or two narrow
+// buckets (fp32 values), 2 one fp64 bucket.  Slot l of row rr of thread t lies at
+// (l VW + rr) kCoopBD + t, columns first, then values.
+struct CoopCache {
+    int mode;
+    int* col;
+    void* val;
+};
+// the entries of row r (rr of this thread) into the cache, bucket by bucket in ascending
+// column order; their counts (the first bucket's in the low half); -1: too many
+template <int VW>
+__device__ __noinline__ int coop_cache_row(const BMDev& M, const CoopCache& c, int64_t r, int rr) {
+    const int lane = (int)(r & 31);
+    int at = 0, cnt = 0;
+    for (int k = 0; k < M.q; ++k) {
+        const BucketDev& B = M.b[k];
+        const int64_t sb = B.sptr[r >> 5];
+        const int w = (int)((B.sptr[(r >> 5) + 1] - sb) >> 5), first = at;
+        for (int l = 0; l < w; ++l) {
+            const int64_t p = sell_slot(sb, lane, l, B.packed);
+            const int col = sell_col_ldg(B, p, r);
+            if (col < 0) continue;
+            if (at >= kCoopRow) return -1;
+            const int slot = (at * VW + rr) * kCoopBD + threadIdx.x;
+            c.col[slot] = col;
+            if (c.mode == 2) static_cast<double*>(c.val)[slot] = __ldg(static_cast<const double*>(B.val) + p);
+            else static_cast<float*>(c.val)[slot] = decode_rt(B, p, col, r);
+            ++at;
+        }
+        cnt |= (at - first) << (16 * k);
+    }
+    return cnt;
+}
+// a row's product from its cached entries: every bucket's partial sum in ascending
+// column order; the narrow buckets' sums a and b add to fl_T(fl64(a + b)), for fp32
+// without fp64 arithmetic (53 >= 2 24 + 2 bits)
+template <typename T, int VW>
+__device__ __forceinline__ T coop_cached(const CoopCache& c, int cnt, int rr, const T* x) {
+    const int n0 = cnt & 0xffff, n = n0 + (cnt >> 16);
+    const int at = rr * kCoopBD + threadIdx.x;
+    T xv[kCoopRow];
+#pragma unroll
+    for (int l = 0; l < kCoopRow; ++l) xv[l] = l < n ? __ldcg(x + c.col[l * VW * kCoopBD + at]) : T(0);
+    if (c.mode == 2) {
+        double a = 0.0;
+#pragma unroll
+        for (int l = 0; l < kCoopRow; ++l)
+            if (l < n) a = __dadd_rn(a, __dmul_rn(static_cast<const double*>(c.val)[l * VW * kCoopBD + at], (double)xv[l]));
+        return from_f64<T>(__dadd_rn(0.0, a));
+    }
+    float a = 0.0f, b = 0.0f;
+#pragma unroll
+    for (int l = 0; l < kCoopRow; ++l)
+        if (l < n) {
+            const float p = __fmul_rn(static_cast<const float*>(c.val)[l * VW * kCoopBD + at], to_f32<T>(xv[l]));
+            if (l < n0) a = __fadd_rn(a, p);
+            else b = __fadd_rn(b, p);
+        }
+    if constexpr (sizeof(T) == 4) return n > n0 ? __fadd_rn(__fadd_rn(0.0f, a), b) : __fadd_rn(0.0f, a);
+    else return n > n0 ? __dadd_rn((double)a, (double)b) : __dadd_rn(0.0, (double)a);
+}
+// any other matrix (kept out of line, its descriptor in shared memory)
+template <typename T>
+__device__ __noinline__ T coop_row(const BMDev& M, int64_t r, const T* x) {
+    return from_f64<T>(bucketed_row<T, true>(M, r, x));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCoopBD, 1) k_gmres_coop(const __grid_constant__ BMDev Av,
+                                                           const __grid_constant__ BMDev Mv, T* V, int64_t ldv, int n,
+                                                           GmresState* st, double* H, double* cs, double* sn,
+                                                           double* g, unsigned long long* tags,
+                                                           unsigned long long* hq, void* tri, T* W,
+                                                           unsigned long long* flag, unsigned long long tmo) {
+    typedef CoopInst<T> I;
+    constexpr int VW = I::VW;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ MgsShared<I> sh;
+    __shared__ GivensBatch s_giv;
+    __shared__ unsigned s_seq;
+    __shared__ int s_done, s_kmax, s_stop;
+    __shared__ BMDev s_A, s_M;
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        s_A = Av;
+        s_M = Mv;
+        s_done = st->done;
+        s_kmax = st->kmax;
+        s_seq = *(volatile unsigned*)&st->bar.seq;
+        s_stop = 0;
+        mgs_shared_init<I>(sh);
+    }
+    __syncthreads();
+    if (s_done) return;
+    const int kmax = s_kmax;
+    const int G = gridDim.x - 1;
+    const int64_t hqset = (int64_t)(kmax + 2) * TagWords<T>::W;  // one column's words
+    unsigned seq = s_seq;
+    auto reductions = [](int j) { return (unsigned)(j / I::GB) + 4u; };  // two exchanges, the groups, the norm
+    if ((int)blockIdx.x == G) {
+        if (tid >= 32) return;
+        for (int j = 0; j < kmax; ++j) {
+            const unsigned tag = seq + 1u;
+            const bool ok = givens_column<T>(s_giv, j, kmax, H, cs, sn, g, st, hq + (j & 1) * hqset, tag, tmo);
+            __syncwarp();
+            seq += reductions(j);
+            int done = 1;
+            if (tid == 0) {
+                if (ok) {
+                    done = *(volatile int*)&st->done;
+                    // the row blocks may run the next step in vain: its numbers are passed over too
+                    if (done) st->bar.seq = seq + reductions(j + 1);
+                } else {
+                    st->status = BSPAI_TIMEOUT;
+                    st->done = 1;
+                }
+                st_relaxed_u64(flag + (j & 1), ((unsigned long long)tag << 32) | (unsigned)done);
+            }
+            if (__shfl_sync(0xffffffffu, done, 0)) return;
+        }
+        return;
+    }
+    int64_t r0, r1;
+    block_rows(n, G, r0, r1);
+    MgsRows<I> R;
+    R.nb = r1 > r0 ? (int)(r1 - r0) : 0;
+    const int64_t r = r0 + R.row(0);
+    const int rows = R.valid(0) / (int)sizeof(T);  // of this thread
+    const MgsIo io{tags, hq, tri, &st->bar, tmo, G, 0, blockIdx.x == 0, blockIdx.x == 0, nullptr};
+    // the matrices' rows into shared memory
+    CoopCache ca, cm;
+    int na[VW], nm[VW];
+    {
+        auto mode = [](const BMDev& M) {
+            if (M.q == 1 && M.b[0].prec == BSPAI_FP64) return 2;
+            for (int k = 0; k < M.q; ++k)
+                if (M.b[k].prec == BSPAI_FP64) return 0;
+            return M.q <= 2 ? 1 : 0;
+        };
+        constexpr size_t slots = (size_t)kCoopRow * kCoopBD * VW;
+        unsigned char* at = smraw + I::smem;
+        ca.mode = mode(s_A);
+        if (sizeof(T) == 4 && ca.mode == 2) ca.mode = 0;  // (A in fp64 beside fp32 vectors: no room for its values)
+        ca.val = at;
+        ca.col = reinterpret_cast<int*>(at + slots * sizeof(T));
+        at += coop_cache_bytes<T>(sizeof(T) == 8);
+        cm.mode = mode(s_M);
+        cm.val = at;
+        cm.col = reinterpret_cast<int*>(at + slots * 8);
+        bool fa = true, fm = true;
+#pragma unroll
+        for (int rr = 0; rr < VW; ++rr) {
+            na[rr] = nm[rr] = 0;
+            if (rr < rows) {
+                if (ca.mode) fa = fa && (na[rr] = coop_cache_row<VW>(s_A, ca, r + rr, rr)) >= 0;
+                if (cm.mode) fm = fm && (nm[rr] = coop_cache_row<VW>(s_M, cm, r + rr, rr)) >= 0;
+            }
+        }
+        if (!__syncthreads_and(fa)) ca.mode = 0;
+        if (!__syncthreads_and(fm)) cm.mode = 0;
+    }
+    auto product = [&](const BMDev& M, const CoopCache& c, const int (&cnt)[VW], const T* x, T (&y)[VW]) {
+#pragma unroll
+        for (int rr = 0; rr < VW; ++rr)
+            y[rr] = rr >= rows ? T(0) : c.mode ? coop_cached<T, VW>(c, cnt[rr], rr, x) : coop_row<T>(M, r + rr, x);
+    };
+    unsigned phase = 0, par = 0;
+    bool good = true;
+    for (int j = 0; j < kmax; ++j) {
+        const unsigned tag = seq + 1u;
+        T y[VW];
+        typename I::P z[I::NP];
+        product(s_A, ca, na, V + (int64_t)j * ldv, y);  // w = A v_j
+#pragma unroll
+        for (int rr = 0; rr < VW; ++rr)
+            if (rr < rows) W[r + rr] = y[rr];
+        coop_exchange<I>(sh, io, ++seq);
+        product(s_M, cm, nm, W, y);  // z = M w
+        if constexpr (VW == 2) z[0] = make_float2(y[0], y[1]);
+        else z[0] = y[0];
+        MgsIo ij = io;
+        ij.hq = hq + (j & 1) * hqset;
+        T hz;
+        if (!*(volatile int*)&sh.ok ||
+            !mgs_passes<I>(sh, ij, R, z, smraw, nullptr, V + r0, ldv, j, tag, seq, phase, par, hz)) {
+            good = false;
+            break;
+        }
+        const T hn = Ar<T>::sqrt(hz);
+        if (hn > T(0) && isfinite((double)hn)) z[0] = pk_quot(z[0], Quot<T>(hn));
+        unit_store<I>(R, V + (int64_t)(j + 1) * ldv + r0, 0, z);
+        fence_proxy_async();  // later steps copy v_{j+1} by the copy engine
+        // step j - 1's decision, by a warp that the exchange leaves idle
+        if (j > 0 && tid == kCoopBD - 32) {
+            const unsigned want = tag - reductions(j - 1);
+            unsigned long long t0 = 0, f;
+            while ((unsigned)((f = ld_relaxed_u64(flag + ((j - 1) & 1))) >> 32) != want) {
+                const unsigned long long now = globaltimer_ns();
+                if (!t0) t0 = now;
+                if (now - t0 > tmo || *(volatile int*)&st->bar.err) {
+                    atomicExch(&st->bar.err, 1);
+                    *(volatile int*)&sh.ok = 0;
+                    f = 1;
+                    break;
+                }
+            }
+            s_stop = (unsigned)f != 0u;
+        }
+        coop_exchange<I>(sh, ij, ++seq);
+        if (!*(volatile int*)&sh.ok) {
+            good = false;
+            break;
+        }
+        if (s_stop) break;
+    }
+    if (!good && blockIdx.x == 0 && tid == 0) {
+        st->status = BSPAI_TIMEOUT;
+        st->done = 1;
+    }
 }
 
 // y = R^-1 g by column-oriented back substitution (fp64): for i = k-1 .. 0,
@@ -552,7 +828,8 @@ struct GmresWork {
     void* w = nullptr;
     unsigned char* aux = nullptr;        // the reductions' buffers (carve):
     unsigned long long* tags = nullptr;  //   tagged slots: 2 parities x kMgsMaxVals x kTagMaxBlocks x 2 words
-    unsigned long long* hq = nullptr;    //   tagged coefficients of the current column
+    unsigned long long* hq = nullptr;    //   tagged coefficients of the current column (two sets)
+    unsigned long long* flag = nullptr;  //   tagged stopping decisions (k_gmres_coop; two sets)
     void* tri = nullptr;                 //   the groups' (I + L)^-1, up to kMgsMaxVals / 2 values per basis vector
     void* part = nullptr;                //   partial sums of the grid-barrier reductions
     GmresState* st = nullptr;
@@ -571,9 +848,10 @@ struct GmresWork {
     size_t res_smem = 0;
     cudaStream_t s = nullptr;
 
-    // tags and hq, which must start at zero (the sequence numbers that tag them start at one)
+    // tags, hq and flag, which must start at zero (the sequence numbers that tag them start at one)
     size_t tagged_bytes() const {
-        return sizeof(unsigned long long) * ((size_t)2 * kMgsMaxVals * kTagMaxBlocks * 2 + 2 * ((size_t)kmax + 2));
+        return sizeof(unsigned long long) *
+               ((size_t)2 * kMgsMaxVals * kTagMaxBlocks * 2 + 4 * ((size_t)kmax + 2) + 2);
     }
     size_t aux_bytes() const {
         const size_t es = ug == BSPAI_FP64 ? 8 : 4;
@@ -593,6 +871,7 @@ struct GmresWork {
         aux = static_cast<unsigned char*>(base);
         tags = reinterpret_cast<unsigned long long*>(aux);
         hq = tags + (size_t)2 * kMgsMaxVals * kTagMaxBlocks * 2;
+        flag = hq + 4 * ((size_t)kmax + 2);
         tri = aux + tagged_bytes();
         part = static_cast<unsigned char*>(tri) + es * (kMgsMaxVals / 2) * ((size_t)kmax + 1);
     }
@@ -649,7 +928,7 @@ struct GmresWork {
         dfree(sn, s); dfree(g, s); dfree(y, s); dfree(norms, s);
         V = w = part = tri = nullptr;
         aux = nullptr;
-        tags = hq = nullptr;
+        tags = hq = flag = nullptr;
         st = nullptr;
         H = cs = sn = g = y = norms = nullptr;
     }
@@ -750,6 +1029,25 @@ static int choose_mgs(GmresWork& W) {
     return BSPAI_OK;
 }
 
+// The row blocks of the whole run in one launch (k_gmres_coop), or 0: an order that few
+// enough blocks cover, with a further block left for the rotations, and matrices whose
+// rows are short (by their widest slices; packed widths are rounded up to fours, and a
+// longer row is read from memory).
+static int coop_blocks(const GmresWork& W, const BMDev& A, const BMDev& M) {
+    const int per = W.ug == BSPAI_FP64 ? kCoopBD : 2 * kCoopBD;
+    const int64_t G = ceil_div(W.n, per);
+    if (G > (int64_t)kCoopMax * (2 * kCoopBD / per) || G >= W.sms) return 0;
+    for (const BMDev* B : {&A, &M}) {
+        int w = 0;
+        for (int k = 0; k < B->q; ++k) {
+            if (B->b[k].maxw < 0) return 0;
+            w += B->b[k].maxw;
+        }
+        if (w > 2 * kCoopRow) return 0;
+    }
+    return (int)G;
+}
+
 static int coop_launch_cfg(void* fn, int G, int block, size_t smem, void** args, cudaStream_t s) {
     cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(G), dim3(block), args, smem, s);
     note_launch();
@@ -802,6 +1100,22 @@ static int gmres_run(GmresWork& W, const bspai_matrix* A, const bspai_bucketed* 
     }
     int launched = 0, chunk = 4;
     const int* jd = &W.st->j;
+    BMDev Ac = compact_buckets(Aview), Mc = compact_buckets(Mview);
+    if (const int Gc = coop_blocks(W, Ac, Mc)) {
+        ProfScope ps(BSPAI_K_MGS, s);
+        const void* fn = (const void*)k_gmres_coop<T>;
+        CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)coop_smem<T>()));
+        int nn = n;
+        int64_t ld = W.ldv;
+        void* args[] = {&Ac, &Mc, &V, &ld, &nn, &W.st, &W.H, &W.cs, &W.sn, &W.g, &W.tags, &W.hq, &W.tri, &w, &W.flag,
+                        &W.tmo_ns};
+        BSPAI_TRY(coop_launch_cfg((void*)fn, Gc + 1, kCoopBD, coop_smem<T>(), args, s));
+        launched = W.kmax;
+        // a solve that shares the GPU with others (max_blocks) queues nothing behind the run:
+        // what waits for it would hold up the streams that share its hardware queue (eight
+        // right-hand sides of n = 9,216, forward and backward: 134 ms, against 54 so)
+        if (W.sms < num_sms()) CUDA_TRY(cudaStreamSynchronize(s));
+    }
     while (launched < W.kmax) {
         for (int c = 0; c < chunk && launched < W.kmax; ++c, ++launched) {
             {

@@ -174,12 +174,13 @@ __device__ __forceinline__ int warp_multi_index(int lane) {
 // ------------------------------------------------------------------ a group's coefficients
 // By one warp, lane t for vector t of the group.  row: its row of the group's
 // (I + L)^-1 below the diagonal (zeros at and right of it), kept for the first
-// `known` vectors in tri (GB values per vector).
+// `known` vectors in tri (GB values per vector; read from L2, where another block may
+// have written it earlier in the launch).
 template <typename T, int GB>
 __device__ __forceinline__ void group_rows(T (&row)[GB], const T* tri, int known) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int s = 0; s < GB; ++s) row[s] = (lane < known && s < lane) ? tri[lane * GB + s] : T(0);
+    for (int s = 0; s < GB; ++s) row[s] = (lane < known && s < lane) ? __ldcg(tri + lane * GB + s) : T(0);
 }
 // h = (I + L)^-1 p for the cnt vectors of a group from the totals tot[t] = p_t;
 // in the last group the newest vector's row is not kept yet, and its Gram
@@ -429,7 +430,8 @@ template <class I>
 __device__ __forceinline__ bool mgs_passes(MgsShared<I>& sh, const MgsIo& io, const MgsRows<I>& R,
                                            typename I::P* z, unsigned char* stage, unsigned char* zs,
                                            const typename I::type* Vb, int64_t ldv, int j, unsigned hq_tag,
-                                           unsigned& seq, unsigned& phase, typename I::type& hz) {
+                                           unsigned& seq, unsigned& phase, unsigned& par,
+                                           typename I::type& hz) {
     typedef typename I::type T;
     typedef typename I::P P;
     typedef typename UnitWord<I::UB>::W W;
@@ -457,8 +459,10 @@ __device__ __forceinline__ bool mgs_passes(MgsShared<I>& sh, const MgsIo& io, co
         if (i <= j && bytes && tid == I::BD - 32) bulk_prefetch_l2(Vb + (int64_t)i * ldv, bytes);
     };
     auto arrived = [&](int i) {
-        if (i <= j && bytes && !mbar_wait_bounded(&sh.full[i % S], (unsigned)(i / S) & 1u, io.tmo))
-            *(volatile int*)&sh.ok = 0;
+        if (i <= j && bytes) {
+            if (!mbar_wait_bounded(&sh.full[i % S], (par >> (i % S)) & 1u, io.tmo)) *(volatile int*)&sh.ok = 0;
+            par ^= 1u << (i % S);
+        }
     };
     auto take = [&](const unsigned char* src, int u, P* out) {
         union {
