@@ -36,12 +36,12 @@ sys.path.insert(0, ROOT)
 METRIC = "GMRES-IR solves/s at fwd err<=1e-10; bucketed M·v GB/s vs GB300 HBM peak"
 UNIT = "solves/s"
 FE_TARGET = 1e-10
-# DRAM bytes over algorithmic bytes of the MGS kernel (k_mgs_res2<16, 512>, z in registers, 128
-# blocks, reductions polled by bulk copies) from one ncu capture of an Arnoldi step (j = 20, 128^3,
-# kmax 64): dram read + write 184.62 + 4.02 = 188.64 MB against (j+1) n 4 + n 4 = 184.55 MB.  Both grow
-# linearly in j, so the per-launch traffic of the timed launches is this ratio times their
+# DRAM bytes over algorithmic bytes of the MGS kernel (k_mgs_res2<16, 512>, z in registers, groups of
+# basis vectors per reduction, 129 blocks) from one ncu capture of an Arnoldi step (j = 20, 128^3,
+# 24 steps): dram read + write 184.63 + 0.38 = 185.01 MB against (j+1) n 4 + n 4 = 184.55 MB.  Both
+# grow linearly in j, so the per-launch traffic of the timed launches is this ratio times their
 # algorithmic bytes.
-MGS_TRAFFIC_RATIO = 188.64 / 184.55
+MGS_TRAFFIC_RATIO = 185.01 / 184.55
 
 
 def parse():
@@ -712,7 +712,7 @@ def main():
         ni = np.diff((Pb @ Ab).tocsr().indptr).astype(np.float64)  # |I_k|: the shadow of J_k
         nj = np.diff(P.row_ptr).astype(np.float64)                  # |J_k|
         spai_flops = float(np.sum(2 * nj ** 2 * (ni - nj / 3) + 4 * ni * nj))
-        res_ops = 10.0 * A.nnz + n  # Dot2: 10 fp64 operations per entry, one add per row
+        res_ops = 7.0 * A.nnz + n  # Dot2: 7 fp64 operations per entry, one add per row
         n_res = ir_steps + len(infos)
         t_spai = prof["spai"][0] / args.steps / 1000.0
         t_res = prof["residual"][0] / (n_res * 1000.0) if n_res else 0.0
@@ -727,7 +727,7 @@ def main():
                                     "peak": p64["fma_per_s"] / 1e9, "unit": "Gop/s fp64",
                                     "frac": res_ops / t_res / p64["fma_per_s"] if t_res else None, "traffic": None,
                                     "ops_per_launch": res_ops,
-                                    "work": "10 fp64 operations per entry (TwoProduct: mul + fma; TwoSum: 6; "
+                                    "work": "7 fp64 operations per entry (TwoProduct: mul + fma; FastTwoSum: 3; "
                                             "error update: 2) and one per row",
                                     "peak_source": "measured: bspai_probe_fma fp64 (one operation per FMA)"}
         out["alu_peaks"] = {"fp32_tflops": p32["flops"] / 1e12, "fp64_gfma_per_s": p64["fma_per_s"] / 1e9,

@@ -34,9 +34,9 @@ every build runs exactly once, no warm-up (launch order: fixed fp32,
 adaptive fp32, fixed half, adaptive half).
 --mgs times GMRES runs of K = 2, 8, 16, 32, 64 steps (tau = 0) on the same
 system and fits the MGS kernel-class time to a K + b P(K), P(K) = sum over the
-steps j < K of the j + 2 grid reductions of step j: a is the cost per Arnoldi
-step outside the reductions (launch, prologue, epilogue), b the cost of one
-reduction pass.
+steps j < K of the j + 1 basis vectors of step j and its norm (j + 2): a is the
+cost per Arnoldi step outside them (launch, prologue, epilogue), b the cost of
+one basis vector (several share one grid reduction).
 """
 from __future__ import annotations
 
