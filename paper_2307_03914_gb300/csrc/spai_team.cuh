@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(BD, MINB) k_spai_team(
         s_stat[0] = s_stat[1] = s_stat[2] = 0;
         s_max = 0.0f;
     }
+    __syncthreads();  // a narrow team's own barriers join a warp only, and its counts may come at any time
     auto team_sync = [&]() {
         if constexpr (wide) __syncthreads();
         else __syncwarp();
