@@ -98,7 +98,9 @@ __device__ __forceinline__ int lower_bound_i32(const int* a, int n, int v) {
 
 // at most 51 registers (five 256-thread blocks per SM): the half instance would
 // otherwise take 60 and fit only four
-template <bool H>
+// LIST: the columns that k_spai_team left, instead of all n (an instance of its own: the list's
+// registers would be spilled in the others)
+template <bool H, bool LIST>
 __global__ void __launch_bounds__(256, 5) k_spai(int n, const int32_t* __restrict__ arp, const int32_t* __restrict__ acol,
                                                const double* __restrict__ aval, const double* __restrict__ d,
                                                const int64_t* __restrict__ msptr, const int32_t* __restrict__ mcol,
@@ -111,12 +113,8 @@ __global__ void __launch_bounds__(256, 5) k_spai(int n, const int32_t* __restric
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-    if (list) {  // the columns k_spai_team left (n: how many the launch covers)
-        if (k >= cnt->n_left) return;
-        k = list[k];
-    } else if (k >= n) {
-        return;
-    }
+    if (k >= n) return;
+    if constexpr (LIST) k = list[k];
 
     // per-warp shared-memory carve-up
     const size_t per_warp = spai_warp_bytes(jmax, lmax, lp2);
@@ -514,7 +512,8 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
         auto attr = [&](const void* fn, size_t bytes) {
             return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         };
-        e = attr(h ? (const void*)k_spai<true> : (const void*)k_spai<false>, smem);
+        e = attr(h ? (const void*)k_spai<true, false> : (const void*)k_spai<false, false>, smem);
+        if (e == cudaSuccess) e = attr((const void*)k_spai<false, true>, smem);
         if (e != cudaSuccess) return fail(cuda_error(e, "spai smem attribute", __FILE__, __LINE__));
         // fp32: the smallest team whose columns and candidates hold every block (its rows are
         // checked per column); half, and larger blocks, a warp per column
@@ -538,7 +537,7 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
                 if (e == cudaSuccess) e = cudaStreamSynchronize(s);
                 if (e != cudaSuccess) return fail(cuda_error(e, "spai columns left", __FILE__, __LINE__));
                 if (nl > 0) {
-                    k_spai<false><<<(unsigned)ceil_div(nl, warps), 32 * warps, smem, s>>>(
+                    k_spai<false, true><<<(unsigned)ceil_div(nl, warps), 32 * warps, smem, s>>>(
                         nl, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
                         (float)spai_eps, uf, jmax, lmax, lp2, cnt, left);
                     note_launch();
@@ -547,7 +546,7 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
                 }
             }
         } else {
-            (h ? k_spai<true> : k_spai<false>)<<<(unsigned)ceil_div(n, warps), 32 * warps, smem, s>>>(
+            (h ? k_spai<true, false> : k_spai<false, false>)<<<(unsigned)ceil_div(n, warps), 32 * warps, smem, s>>>(
                 n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
                 (float)spai_eps, uf, jmax, lmax, lp2, cnt, nullptr);
             note_launch();
