@@ -44,18 +44,97 @@ int launch_row_absmax_inv(int n, const int32_t* row_ptr, const double* val, doub
     return BSPAI_OK;
 }
 
-// per column: |J_k| and the candidate count sum_{j in J_k} |row j of A|
+// Which form solves a column's block depends on how many distinct rows its candidates come to;
+// the limits that the choice asks about (team_pays), and the candidates up to which it does
+constexpr int kNarrowRows = 32, kTallRows = 96, kWideLeast = 196, kSampleL = 256;
+
+// |I_k| of a column by a warp, from its row of M at base: the distinct columns among its
+// candidates, eight per lane (at most kSampleL; |J| <= 32).  Above `enough`, any larger number.
+__device__ __forceinline__ int shadow_rows(int64_t base, int nJ, int enough, const int32_t* __restrict__ mcol,
+                                           const int32_t* __restrict__ arp, const int32_t* __restrict__ acol) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int E = kSampleL / 32;
+    const int lane = threadIdx.x & 31;
+    int rb = 0, len = 0;
+    if (lane < nJ) {
+        const int j = mcol[base + (int64_t)lane * kSlice];
+        rb = arp[j];
+        len = arp[j + 1] - rb;
+    }
+    int end = len;  // entries of rows J up to and with this lane's
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(full, end, o);
+        if (lane >= o) end += v;
+    }
+    const int L = __shfl_sync(full, end, 31);
+    int c[E];
+    bool fresh[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        c[e] = -1;
+        if (32 * e >= L) continue;
+        // candidate idx is entry idx - (end - len) of the row whose entries end above it
+        const int idx = lane + 32 * e;
+        int at = -1;
+        for (int q = 0; q < nJ; ++q) {
+            const int hi = __shfl_sync(full, end, q), first = __shfl_sync(full, rb - (end - len), q);
+            if (at < 0 && idx < hi) at = first + idx;
+        }
+        if (at >= 0) c[e] = acol[at];
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) fresh[e] = c[e] >= 0;
+    int nI = 0;  // among the first 32 (e0 + 1) candidates
+#pragma unroll
+    for (int e0 = 0; e0 < E; ++e0) {
+        if (32 * e0 >= L || nI > enough) break;
+#pragma unroll 4
+        for (int l = 0; l < 32; ++l) {
+            const int v = __shfl_sync(full, c[e0], l);  // (an absent one, -1, meets none that is fresh)
+            if (lane > l && c[e0] == v) fresh[e0] = false;
+#pragma unroll
+            for (int e = e0 + 1; e < E; ++e)
+                if (c[e] == v) fresh[e] = false;
+        }
+        nI += __popc(__ballot_sync(full, fresh[e0]));
+    }
+    return nI;
+}
+
+// Per column: |J_k| and the candidate count sum_{j in J_k} |row j of A|; their maxima go to
+// out[0], out[1].  One column per warp of every `every`-th block (0: none) is looked at further: out[2]
+// counts these, out[3] and out[4] those with more than kNarrowRows and kTallRows distinct rows.
 __global__ void __launch_bounds__(256) k_spai_sizes(int n, const int64_t* __restrict__ msptr, const int32_t* __restrict__ mcol,
                              const int32_t* __restrict__ mrowlen, const int32_t* __restrict__ arp,
-                             int* __restrict__ out) {
+                             const int32_t* __restrict__ acol, int every, int* __restrict__ out) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t base = k < n ? msptr[k >> 5] + (k & 31) : 0;
     int nJ = 0, L = 0;
     if (k < n) {
         nJ = mrowlen[k];
-        const int64_t base = msptr[k >> 5] + (k & 31);
         for (int q = 0; q < nJ; ++q) {
             const int j = mcol[base + (int64_t)q * kSlice];
             L += arp[j + 1] - arp[j];
+        }
+    }
+    if (every > 0 && blockIdx.x % every == 0) {
+        // the warp's column: another lane in each warp, so that no period of the rows is met
+        const int src = (int)((blockIdx.x * 8u + (threadIdx.x >> 5)) * 2654435761u >> 27);
+        const int sj = __shfl_sync(0xffffffffu, nJ, src), sl = __shfl_sync(0xffffffffu, L, src);
+        const int64_t sb = __shfl_sync(0xffffffffu, base, src);
+        const bool in = __shfl_sync(0xffffffffu, (int)(k < n), src) != 0;
+        int rows = sl;
+        if (in && sl > kNarrowRows && sl <= kSampleL && sj <= 32)
+            rows = shadow_rows(sb, sj, sl < kWideLeast ? kNarrowRows : kTallRows, mcol, arp, acol);
+        // the block's three counts in one word
+        __shared__ int s_seen[8];
+        const int seen = block_combine(!in ? 0 : 1 + (rows > kNarrowRows ? 1 << 8 : 0) + (rows > kTallRows ? 1 << 16 : 0),
+                                       0, s_seen, [](int a, int b) { return a + b; });
+        if (threadIdx.x == 0) {
+            atomicAdd(out + 2, seen & 255);
+            if (seen >> 8) atomicAdd(out + 3, (seen >> 8) & 255);
+            if (seen >> 16) atomicAdd(out + 4, seen >> 16);
         }
     }
     // the warp's maxima, then the block's, then one atomic each
@@ -400,6 +479,22 @@ static const SpaiTeamKernel kSpaiTeams[] = {
     spai_team<8, 16, 4, 12, 256, 2>(),  // 9-point: |J| <= 12, 128 candidates, 32 rows
     spai_team<128, 4, 4, 24, 128, 4>(), // |J| <= 24, 512 candidates and rows
 };
+// Whether an instance that could hold the blocks is faster than a warp per column, from a sample
+// of the columns (seen: [0] how many, [1] with more than kNarrowRows distinct rows, [2] with more
+// than kTallRows).  Measured at n = 65,536 (us, warp per column -> team):
+//   narrow: pays while at most half of the columns are too tall for it and are solved by k_spai
+//     after it.  None: 7-point 369 -> 258, 9-point 676 -> 342; a quarter 419 -> 373, 707 -> 509;
+//     half 471 -> 469, 731 -> 668; three quarters 519 -> 558, 769 -> 809; all (|J| scattered
+//     entries per row, 7 or 11) 569 -> 644, 1,337 -> 1,501.
+//   wide: a block of 128 threads takes as long for a low shadow as for a tall one, a warp does
+//     not, and the warps' shared memory leaves few of them on an SM above 256 candidates.  144 to
+//     169 candidates: 1,508 to 2,299 -> 3,592 to 3,764; 196 to 256: 3,200 to 3,813 -> 3,841 to
+//     4,085 on bands (27 to 31 distinct rows), 4,761 to 6,843 -> 3,887 to 4,124 on scattered
+//     rows (about 190 to 250); 289: 9,011 -> 4,204 and 14,583 -> 4,282.
+static bool team_pays(const SpaiTeamKernel& c, int lmax, const int* seen) {
+    if (c.rows < c.slots) return lmax <= c.rows || (seen[0] > 0 && 2 * (int64_t)seen[1] <= seen[0]);
+    return lmax > kSampleL || (lmax >= kWideLeast && 2 * (int64_t)seen[2] > seen[0]);
+}
 
 // fp64 values rounded once to fp16 (held in fp64), for an M imported in u_f = fp16
 __global__ void k_round_f16_of_f64(int64_t n, const double* __restrict__ x, double* __restrict__ y) {
@@ -470,25 +565,29 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
         if ((st_ = dalloc_t(&M->val, (size_t)M->sell.slots, s))) return fail(st_);
         if ((st_ = dalloc_t(&M->resid, (size_t)n, s))) return fail(st_);
         if ((st_ = dalloc_t(&d, (size_t)n, s))) return fail(st_);
-        if ((st_ = dalloc_t(&sizes, 2, s))) return fail(st_);
+        if ((st_ = dalloc_t(&sizes, 5, s))) return fail(st_);
         if ((st_ = dalloc_t(&cnt, 1, s))) return fail(st_);
         cudaError_t e = cudaMemcpyAsync(M->csr_row_ptr, P->row_ptr, sizeof(int32_t) * ((size_t)n + 1),
                                         cudaMemcpyDeviceToDevice, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(M->val, 0, sizeof(float) * (size_t)M->sell.slots, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(sizes, 0, 2 * sizeof(int), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(sizes, 0, 5 * sizeof(int), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(SpaiCounters), s);
         if (e != cudaSuccess) return fail(cuda_error(e, "bspai_build setup", __FILE__, __LINE__));
         if (n > 0) {
             k_row_absmax_inv<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(n, A->row_ptr, A->val, d);
             note_launch();
-            k_spai_sizes<<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(n, M->sell.sptr, M->sell.col, M->rowlen,
-                                                                    A->row_ptr, sizes);
+            const int blocks = (int)ceil_div(n, 256);
+            // about 2,048 columns of a large system are looked at further; none where it would cost what
+            // a team gives (5 to 8 us; at 3,600 rows a 9-point build takes 205 us in either form)
+            const int every = u_f != BSPAI_FP32 || n <= 8192 ? 0 : blocks <= 256 ? 1 : blocks / 256;
+            k_spai_sizes<<<(unsigned)blocks, 256, 0, s>>>(n, M->sell.sptr, M->sell.col, M->rowlen, A->row_ptr, A->col,
+                                                          every, sizes);
             note_launch();
             e = cudaGetLastError();
             if (e != cudaSuccess) return fail(cuda_error(e, "spai sizes", __FILE__, __LINE__));
         }
     }
-    int hs[2] = {0, 0};
+    int hs[5] = {0, 0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(hs, sizes, sizeof hs, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(cuda_error(e, "spai sizes copy", __FILE__, __LINE__));
@@ -505,58 +604,52 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
                               "bspai_build: least-squares blocks too large (|J| <= %d, candidates <= %d need %zu bytes)",
                               jmax, lmax, per_warp));
     const size_t smem = per_warp * warps;
-    if (n > 0) {
+    const bool h = u_f == BSPAI_FP16;
+    const float uf = h ? 4.8828125e-04f : 5.9604644775390625e-08f;  // 2^-11 or 2^-24, the rank test's unit roundoff
+    auto attr = [&](const void* fn, size_t bytes) {
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    auto warp_per_column = [&](auto kern, int count, const int* list) {
         ProfScope ps(BSPAI_K_SPAI, s);
-        const bool h = u_f == BSPAI_FP16;
-        const float uf = h ? 4.8828125e-04f : 5.9604644775390625e-08f;  // 2^-11 or 2^-24, the rank test's unit roundoff
-        auto attr = [&](const void* fn, size_t bytes) {
-            return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        };
-        e = attr(h ? (const void*)k_spai<true, false> : (const void*)k_spai<false, false>, smem);
-        if (e == cudaSuccess) e = attr((const void*)k_spai<false, true>, smem);
-        if (e != cudaSuccess) return fail(cuda_error(e, "spai smem attribute", __FILE__, __LINE__));
-        // fp32: the smallest team whose columns and candidates hold every block (its rows are
-        // checked per column); half, and larger blocks, a warp per column
-        const SpaiTeamKernel* tk = nullptr;
-        if (!h)
-            for (const SpaiTeamKernel& c : kSpaiTeams)
-                if (!tk && jmax <= c.cols && lmax <= c.slots) tk = &c;
-        if (tk) {
-            if ((st_ = dalloc_t(&left, (size_t)n, s))) return fail(st_);
-            e = attr((const void*)tk->fn, tk->smem);
-            if (e != cudaSuccess) return fail(cuda_error(e, "spai team smem attribute", __FILE__, __LINE__));
-            tk->fn<<<(unsigned)ceil_div(n, tk->per_block), tk->threads, tk->smem, s>>>(
-                n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
-                (float)spai_eps, uf, cnt, left);
-            note_launch();
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return fail(cuda_error(e, "k_spai_team", __FILE__, __LINE__));
-            if (lmax > tk->rows) {  // a shadow could be larger than the team's rows
-                int nl = 0;
-                e = cudaMemcpyAsync(&nl, &cnt->n_left, sizeof nl, cudaMemcpyDeviceToHost, s);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-                if (e != cudaSuccess) return fail(cuda_error(e, "spai columns left", __FILE__, __LINE__));
-                if (nl > 0) {
-                    k_spai<false, true><<<(unsigned)ceil_div(nl, warps), 32 * warps, smem, s>>>(
-                        nl, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
-                        (float)spai_eps, uf, jmax, lmax, lp2, cnt, left);
-                    note_launch();
-                    e = cudaGetLastError();
-                    if (e != cudaSuccess) return fail(cuda_error(e, "k_spai", __FILE__, __LINE__));
-                }
-            }
-        } else {
-            (h ? k_spai<true, false> : k_spai<false, false>)<<<(unsigned)ceil_div(n, warps), 32 * warps, smem, s>>>(
-                n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
-                (float)spai_eps, uf, jmax, lmax, lp2, cnt, nullptr);
-            note_launch();
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return fail(cuda_error(e, "k_spai", __FILE__, __LINE__));
-        }
-    }
+        cudaError_t e2 = attr((const void*)kern, smem);
+        if (e2 != cudaSuccess) return e2;
+        kern<<<(unsigned)ceil_div(count, warps), 32 * warps, smem, s>>>(
+            count, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
+            (float)spai_eps, uf, jmax, lmax, lp2, cnt, list);
+        note_launch();
+        return cudaGetLastError();
+    };
     SpaiCounters hc{};
-    e = cudaMemcpyAsync(&hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    auto counters = [&]() {
+        cudaError_t e2 = cudaMemcpyAsync(&hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, s);
+        return e2 == cudaSuccess ? cudaStreamSynchronize(s) : e2;
+    };
+    // fp32: the first instance that holds every block's columns and candidates and is the faster
+    // one for these shadows (team_pays); half, larger blocks and the rest, a warp per column
+    const SpaiTeamKernel* tk = nullptr;
+    if (!h && n > 0)
+        for (const SpaiTeamKernel& c : kSpaiTeams)
+            if (!tk && jmax <= c.cols && lmax <= c.slots && team_pays(c, lmax, hs + 2)) tk = &c;
+    if (tk) {
+        ProfScope ps(BSPAI_K_SPAI, s);
+        if ((st_ = dalloc_t(&left, (size_t)n, s))) return fail(st_);
+        e = attr((const void*)tk->fn, tk->smem);
+        if (e != cudaSuccess) return fail(cuda_error(e, "spai team smem attribute", __FILE__, __LINE__));
+        tk->fn<<<(unsigned)ceil_div(n, tk->per_block), tk->threads, tk->smem, s>>>(
+            n, A->row_ptr, A->col, A->val, d, M->sell.sptr, M->sell.col, M->rowlen, M->val, M->resid,
+            (float)spai_eps, uf, cnt, left);
+        note_launch();
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return fail(cuda_error(e, "k_spai_team", __FILE__, __LINE__));
+    } else if (n > 0) {
+        e = h ? warp_per_column(k_spai<true, false>, n, nullptr) : warp_per_column(k_spai<false, false>, n, nullptr);
+        if (e != cudaSuccess) return fail(cuda_error(e, "k_spai", __FILE__, __LINE__));
+    }
+    e = counters();
+    if (e == cudaSuccess && hc.n_left > 0) {  // columns taller than their team
+        e = warp_per_column(k_spai<false, true>, hc.n_left, left);
+        if (e == cudaSuccess) e = counters();
+    }
     if (e != cudaSuccess) return fail(cuda_error(e, "spai counters", __FILE__, __LINE__));
     dfree(d, s);
     dfree(sizes, s);

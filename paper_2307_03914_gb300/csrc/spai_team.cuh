@@ -321,16 +321,17 @@ __global__ void __launch_bounds__(BD, MINB) k_spai_team(
     };
     fro = __fsqrt_rn(one_sum(fro));
     float rd[NC];
+    const int nS = work ? nJ : 0;  // steps of this column (none: left to k_spai)
     auto step = [&](auto C) {
         constexpr int c = decltype(C)::value;
         constexpr int pr = c / TS, pl = c % TS;  // the thread and register of row c
         rd[c] = 1.0f;
         if constexpr (wide) {
-            if (c >= nJ) return;  // (the whole block)
+            if (c >= nS) return;  // (the whole block)
         } else {
-            if (__all_sync(full, c >= nJ)) return;
+            if (__all_sync(full, c >= nS)) return;
         }
-        const bool act = c < nJ && !rankdef;
+        const bool act = c < nS && !rankdef;
         float x[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) x[r] = (TS * (r + 1) <= c || (TS * r < c && t + TS * r < c)) ? 0.0f : a[r][c];

@@ -43,7 +43,7 @@ def _matrices(n, width, run):
 @pytest.mark.parametrize("run", [1, 4, 32])
 def test_counts_match_the_columns(width, run):
     B = lib()
-    A, P = _matrices(6000, width, run)
+    A, P = _matrices(8500, width, run)
     eps = 0.2
     for rep in range(8):
         g = gpu_build(B, dict(A=A, pattern=P, spai_eps=eps))
