@@ -118,6 +118,51 @@ __global__ void __launch_bounds__(512) k_gmres_start(T* __restrict__ V, int n, G
 // (fp64 keeps one block per SM: the grid, which k_gmres_start shares, fixes the
 // order in which ||M r||_2 is summed.)
 constexpr int kStreamGB = 4;
+// One sweep of a pass over the block's rows: HAVE vectors from Vp (coefficients hp) out of z,
+// then the products with CNT vectors from Vc, and for the last group (last) the Gram entries
+// of its last vector; CNT = 0: ||z||^2 into a[0].  The counts are constants: no operation is
+// spent on a vector that is not there, and the loads of RT rows are issued ahead of the store
+// that they could not pass.  One loop for every count, a row at a time -> this, us in this
+// kernel: n = 30,000 in fp64 on one SM, the first step 284 (one vector at a time: 223) -> 168;
+// n = 4,000,001 in fp32, the first step 73 (49) -> 49, 30 steps 5,290 (8,254) -> 4,240.
+template <typename T, int HAVE, int CNT>
+__device__ __forceinline__ void stream_sweep(const T* Vp, const T* Vc, int64_t ldv, T* z, int64_t r0, int64_t r1,
+                                             bool last, const T (&hp)[kStreamGB], T (&a)[kStreamGB],
+                                             T (&q)[kStreamGB]) {
+    constexpr int RT = HAVE + CNT <= 2 ? 4 : 2;
+    const int64_t bd = blockDim.x;
+    for (int64_t rb = r0 + threadIdx.x; rb < r1; rb += RT * bd) {
+        T zr[RT], pv[RT][HAVE ? HAVE : 1], v[RT][CNT ? CNT : 1];
+#pragma unroll
+        for (int u = 0; u < RT; ++u) {
+            const int64_t r = rb + u * bd;
+            const bool in = r < r1;
+            zr[u] = in ? z[r] : T(0);
+#pragma unroll
+            for (int t = 0; t < HAVE; ++t) pv[u][t] = in ? Vp[(int64_t)t * ldv + r] : T(0);
+#pragma unroll
+            for (int t = 0; t < CNT; ++t) v[u][t] = in ? Vc[(int64_t)t * ldv + r] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < RT; ++u) {
+            if (rb + u * bd >= r1) break;
+            if constexpr (HAVE > 0) {
+#pragma unroll
+                for (int t = 0; t < HAVE; ++t) zr[u] = pk_nfma(hp[t], pv[u][t], zr[u]);
+                z[rb + u * bd] = zr[u];
+            }
+            if constexpr (CNT == 0) {
+                a[0] = Ar<T>::fma(zr[u], zr[u], a[0]);
+            } else {
+#pragma unroll
+                for (int t = 0; t < CNT; ++t) a[t] = Ar<T>::fma(v[u][t], zr[u], a[t]);
+                if (last)
+#pragma unroll
+                    for (int t = 0; t < CNT - 1; ++t) q[t] = Ar<T>::fma(v[u][t], v[u][CNT - 1], q[t]);
+            }
+        }
+    }
+}
 template <typename T>
 __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_mgs(T* __restrict__ V, int64_t ldv, int n, GmresState* st, double* H,
                                              double* cs, double* sn, double* g, T* part, T* tri,
@@ -150,37 +195,27 @@ __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_mgs(T* __restri
         const bool last = gi == ng - 1, norm = gi == ng;
         const int cnt = norm ? 0 : last ? j - i0 + 1 : GB;
         const int have = gi > 0 ? (norm ? j + 1 - (i0 - GB) : GB) : 0;  // vectors of the previous group
-        T a[GB], q[GB], zz = T(0);
+        T a[GB], q[GB];
 #pragma unroll
         for (int t = 0; t < GB; ++t) a[t] = q[t] = T(0);
-        for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-            T v[GB], pv[GB];
-            T zr = z[r];
-#pragma unroll
-            for (int t = 0; t < GB; ++t) {
-                pv[t] = t < have ? V[(int64_t)(i0 - GB + t) * ldv + r] : T(0);
-                v[t] = t < cnt ? V[(int64_t)(i0 + t) * ldv + r] : T(0);
-            }
-            if (have) {
-#pragma unroll
-                for (int t = 0; t < GB; ++t) zr = pk_nfma(hp[t], pv[t], zr);
-                z[r] = zr;
-            }
-            if (norm) {
-                zz = Ar<T>::fma(zr, zr, zz);
-            } else {
-                T vj = v[0];
-#pragma unroll
-                for (int t = 1; t < GB; ++t)
-                    if (t == cnt - 1) vj = v[t];
-#pragma unroll
-                for (int t = 0; t < GB; ++t) {
-                    a[t] = Ar<T>::fma(v[t], zr, a[t]);
-                    if (last) q[t] = Ar<T>::fma(v[t], vj, q[t]);
-                }
-            }
+        const T *Vp = V + (int64_t)(i0 - GB) * ldv, *Vc = V + (int64_t)i0 * ldv;
+        static_assert(GB == 4, "the counts below");
+        if (norm) {
+            if (have == 1) stream_sweep<T, 1, 0>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else if (have == 2) stream_sweep<T, 2, 0>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else if (have == 3) stream_sweep<T, 3, 0>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else stream_sweep<T, 4, 0>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+        } else if (have == 0) {
+            if (cnt == 1) stream_sweep<T, 0, 1>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else if (cnt == 2) stream_sweep<T, 0, 2>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else if (cnt == 3) stream_sweep<T, 0, 3>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else stream_sweep<T, 0, 4>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+        } else {
+            if (cnt == 1) stream_sweep<T, 4, 1>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else if (cnt == 2) stream_sweep<T, 4, 2>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else if (cnt == 3) stream_sweep<T, 4, 3>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
+            else stream_sweep<T, 4, 4>(Vp, Vc, ldv, z, r0, r1, last, hp, a, q);
         }
-        if (norm) a[0] = zz;
         warp_multi_sum<GB>(a);
         warp_multi_sum<GB>(q);
         if ((lane & (32 / GB - 1)) == 0) {
@@ -226,7 +261,14 @@ __global__ void __launch_bounds__(512, sizeof(T) == 8 ? 1 : 2) k_mgs(T* __restri
     const T hn = Ar<T>::sqrt(s_tot[0]);
     if (hn > T(0) && isfinite((double)hn)) {
         const Quot<T> by(hn);
-        for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) z[r] = by(z[r]);
+        for (int64_t rb = r0 + threadIdx.x; rb < r1; rb += 4 * (int64_t)blockDim.x) {
+            T x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = rb + u * blockDim.x < r1 ? z[rb + u * blockDim.x] : T(0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (rb + u * blockDim.x < r1) z[rb + u * blockDim.x] = by(x[u]);
+        }
     }
     if (blockIdx.x == 0 && w == 0) {
         if (lane == 0) {
