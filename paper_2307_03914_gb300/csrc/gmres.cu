@@ -1033,8 +1033,15 @@ static int choose_mgs(GmresWork& W) {
     int Gr = (int)ceil_div(W.n, cap);
     if (Gr < kMgsBlocks) Gr = kMgsBlocks;
     // the Givens block wants an SM of its own (one block per SM at these sizes): the
-    // rotations of a column otherwise follow its last reduction
-    if (Gr >= W.sms) Gr = W.sms > 1 && ceil_div(W.n, W.sms - 1) <= cap ? W.sms - 1 : W.sms;
+    // rotations of a column otherwise follow its last reduction.  Not in fp64 on a few SMs,
+    // where the rows' share of that SM costs more (40 steps, us, with an SM for the rotations
+    // -> without: 2 SMs, 7,505 rows 8,181 -> 5,594; 6, 37,505 8,602 -> 7,877; 12, 22,005
+    // 3,889 -> 3,875; 16, 30,005 3,901 -> 3,953; 38, 74,005 4,021 -> 4,113)
+    if (Gr >= W.sms) {
+        const int64_t share = W.sms > 1 ? ceil_div(W.n, W.sms - 1) : cap + 1;
+        const bool rows_first = W.ug == BSPAI_FP64 && W.sms <= 12 && share > 1024;
+        Gr = share <= cap && !rows_first ? W.sms - 1 : W.sms;
+    }
     if (Gr > kTagMaxBlocks) return BSPAI_OK;
     int64_t chunk = ceil_div(ceil_div(W.n, Gr), 32) * 32;
     const size_t es = W.ug == BSPAI_FP64 ? 8 : 4;
