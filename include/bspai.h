@@ -488,7 +488,7 @@ typedef struct {
     int32_t grid;           /* CTAs of the persistent GMRES launch */
     int32_t kmax;           /* GMRES steps allowed per refinement step */
     int32_t mgs_rows;       /* the schedule's MGS load tile (bspai_batch_schedule_t) */
-    int32_t z_shared_rows;  /* the schedule's z-in-shared-memory limit */
+    int32_t z_shared_rows;  /* the z-in-shared-memory limit that the launches ran with */
     int32_t m_schedule;     /* the schedule's bucket order */
     int32_t team_rows;      /* the schedule's team mode (0: one CTA per pair) */
     int32_t tuned_candidates; /* schedules timed by this call (0: cached or forced) */
@@ -513,7 +513,8 @@ typedef struct {
  *                  orthogonalised, in shared memory for the whole Arnoldi step
  *                  (0 = never; -1 = as many rows as fit); limited by the
  *                  shared memory left at the CTAs per SM that the registers
- *                  allow.
+ *                  allow (a value up to about 1,100 rows (fp64: 800) above it is
+ *                  lowered to it; the solve's info reports what was given).
  *   m_schedule     the bucket schedule of the M products: 0 row-fused (each
  *                  thread takes two rows at a time through every bucket), 1
  *                  bucket-major (one sweep over the pair's rows per bucket,

@@ -1030,8 +1030,8 @@ static int occupancy_blocks(BatchKernel<T> kern, int bd, size_t smem, int* occ) 
 // the most rows a schedule may name (`most`: the SM's shared memory among those CTAs,
 // less 1 KB per CTA that the system reserves and the small static part that has
 // always been set aside) and the most a launch gives (`fit`: what the kernel's own
-// static part leaves; a pair between the two keeps z in memory).  Raises the kernel's
-// dynamic shared memory limit to the opt-in maximum on the way.
+// static part leaves; a schedule that names more is given that, and reported with it).
+// Raises the kernel's dynamic shared memory limit to the opt-in maximum on the way.
 template <typename T>
 static int zcap_limit(BatchKernel<T> kern, int bd, int* most, int* fit) {
     constexpr int kStaticPart = sizeof(T) == 4 ? 416 : 552;
@@ -1188,14 +1188,9 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
     auto zlim = [&](const Sched& c, const int (&t)[2][2][3]) {
         return t[c.urows == MgsU<T>::hi ? 1 : 0][c.msched ? 1 : 0][c.bd == 512 ? 2 : c.bd == 256 ? 1 : 0];
     };
-    auto zfit = [&](const Sched& c) { return zlim(c, zmost); };
-    auto launch_z = [&](const Sched& c) {
-        const int z = zlim(c, zgive);
-        return c.zcap < z ? c.zcap : z;
-    };
     auto grid_for = [&](const Sched& c, int* grid) -> int {
         int occ = 0;
-        int r2 = occupancy_blocks<T>(batch_kernel<T>(c.urows, c.msched), c.bd, sizeof(T) * (size_t)launch_z(c), &occ);
+        int r2 = occupancy_blocks<T>(batch_kernel<T>(c.urows, c.msched), c.bd, sizeof(T) * (size_t)c.zcap, &occ);
         if (r2) return r2;
         if (occ < 1) return set_error(BSPAI_ERR_CUDA, "batched GMRES kernel does not fit on an SM");
         const size_t per = sizeof(T) * (size_t)ldv * (kmax + 2) + sizeof(double) * (size_t)ldv +
@@ -1211,7 +1206,7 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
     };
     // the candidate the tuner tries: every pair of the batch, if it fits
     auto zlimit = [&](const Sched& c) {
-        const int z = zfit(c);
+        const int z = zlim(c, zgive);
         return z < nmax32 ? z : nmax32;
     };
     Sched sch;
@@ -1227,12 +1222,12 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
         if (sch.team > 0 && sizeof(T) != 4)
             return done(set_error(BSPAI_ERR_UNSUPPORTED, "batch schedule: team mode needs u_g = FP32"));
         if (sch.zcap < 0) sch.zcap = zlimit(sch);  // as many rows as fit
-        if (sch.zcap > zfit(sch))
+        if (sch.zcap > zlim(sch, zmost))
             return done(set_error(BSPAI_ERR_INVALID,
                                   "batch schedule: z_shared_rows %d exceeds the %d rows that fit in shared memory "
                                   "at this CTA size and tile",
-                                  sch.zcap, zfit(sch)));
-        if (sch.zcap > nmax32) sch.zcap = nmax32;  // no pair is larger: the same schedule
+                                  sch.zcap, zlim(sch, zmost)));
+        if (sch.zcap > zlimit(sch)) sch.zcap = zlimit(sch);  // what the launch gives; no pair is larger than nmax32
         have = true;
     } else {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -1252,7 +1247,7 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
                     cs.bd = cand_bd[c];
                     cs.urows = u ? MgsU<T>::hi : MgsU<T>::lo;
                     cs.msched = m;
-                    cs.zcap = zs ? (zmost[u][m][c] < nmax32 ? zmost[u][m][c] : nmax32) : 0;
+                    cs.zcap = zs ? zlimit(cs) : 0;
                     int gr;
                     if ((rc = grid_for(cs, &gr))) return done(rc);
                     gmax_all = gr > gmax_all ? gr : gmax_all;
@@ -1275,9 +1270,9 @@ static int batch_ir(bspai_matrix* A, const int32_t* row_off, int nsys, int nrhs,
     if ((rc = take((void**)&d_work, 2 * sizeof(unsigned long long)))) return done(rc);
     auto launch_gmres = [&](const Sched& c, int grid, const double* Rin, double* Xout, int kcap, double tcap,
                             PairState& St, cudaStream_t st, int np) {
-        batch_kernel<T>(c.urows, c.msched)<<<grid, c.bd, sizeof(T) * (size_t)launch_z(c), st>>>(
+        batch_kernel<T>(c.urows, c.msched)<<<grid, c.bd, sizeof(T) * (size_t)c.zcap, st>>>(
             Av, Mv, row_off, nsys, n, d_order, np, d_queue, St.status, Rin, Xout, Vws, Wws, Yws, ldv, Hws, Sws,
-            Tws, kcap, tcap, launch_z(c), St.iters, St.steps, St.relres, St.dmax, St.dxmax, d_work);
+            Tws, kcap, tcap, c.zcap, St.iters, St.steps, St.relres, St.dmax, St.dxmax, d_work);
         note_launch();
         return cudaGetLastError();
     };
