@@ -179,6 +179,13 @@ void bspai_opts_default(bspai_opts_t* opts);
  * Allocates and frees a small device buffer. */
 int bspai_probe_fma(bspai_prec_t prec, int32_t iters, bspai_stream_t s, double* fma_per_s, float* ms);
 
+/* q_i = a_i / h_i (device arrays of n values in prec, BSPAI_FP32 or BSPAI_FP64)
+ * as the Gram-Schmidt kernels form the entries of a new basis vector: from the
+ * rounded reciprocal of h with one correction, within 1/2 + 2^-22 (fp64: 1/2 +
+ * 2^-51) units in the last place, or, outside the range where that holds, by
+ * division.  For tests; no counterpart in the paper. */
+int bspai_probe_quotients(bspai_prec_t prec, int32_t n, const void* a, const void* h, void* q, bspai_stream_t s);
+
 /* Releases any handle returned by this library (NULL is a no-op).  Enqueues
  * the frees on the stream the handle was created on. */
 int bspai_free(void* handle);

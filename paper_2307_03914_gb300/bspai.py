@@ -129,6 +129,7 @@ _sig("bspai_M_transpose", _i, [_vp, _vp, C.POINTER(_vp)])
 _sig("bspai_bucket_transpose", _i, [_vp, _vp, C.POINTER(_vp)])
 _sig("bspai_adjoint_grad_A", _i, [C.POINTER(CsrT), C.c_int32, _vp, _vp, _vp, _vp])
 _sig("bspai_probe_fma", _i, [_i, C.c_int32, _vp, C.POINTER(C.c_double), C.POINTER(C.c_float)])
+_sig("bspai_probe_quotients", _i, [_i, C.c_int32, _vp, _vp, _vp, _vp])
 
 
 _sig("bspai_apply_cw", _i, [_vp, _d, C.POINTER(C.c_int32), C.c_int32, _vp, _i, _vp, _i, _vp,
@@ -456,6 +457,17 @@ def probe_fma(prec="fp32", iters=4096, stream=None) -> dict:
     r, ms = C.c_double(0.0), C.c_float(0.0)
     _check(_lib.bspai_probe_fma(PREC[prec], iters, _stream(stream), C.byref(r), C.byref(ms)))
     return dict(fma_per_s=r.value, flops=2.0 * r.value, ms=ms.value)
+
+
+def probe_quotients(a, h, stream=None):
+    """a / h (device tensors, both fp32 or both fp64) as the Gram-Schmidt kernels form it (for tests)."""
+    if a.dtype != h.dtype or a.shape != h.shape or a.dtype not in (torch.float32, torch.float64):
+        raise ValueError("probe_quotients: two fp32 or two fp64 tensors of one shape")
+    a, h = a.contiguous(), h.contiguous()
+    q = torch.empty_like(a)
+    _check(_lib.bspai_probe_quotients(PREC["fp32" if a.dtype == torch.float32 else "fp64"], a.numel(), _ptr(a), _ptr(h),
+                                      _ptr(q), _stream(stream)))
+    return q
 
 
 def apply_cw(M: MHandle, bucket_eps: float, precs, x, y, ids=None, counts=False, stream=None):

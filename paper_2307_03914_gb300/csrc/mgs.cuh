@@ -117,19 +117,33 @@ __device__ __forceinline__ float pk_sum(float2 a) { return __fadd_rn(a.x, a.y); 
 // a / h for many a and one h, from its rounded reciprocal r: the quotient a r
 // corrected once by its residual (Markstein, "Computation of elementary functions
 // on the IBM RISC System/6000 processor", 1990), three operations where a division
-// takes a dozen on the narrow fp64 pipe.  An h whose reciprocal or residuals could
-// leave the format's range is divided by.
+// takes a dozen on the narrow fp64 pipe.  With r = (1 + d1) / h, q = (1 + d2) a r and
+// the residual rounded once (d3), all |d| <= u = 2^-24 or 2^-53, what is rounded last
+// differs from a / h by (2 u) (2 u) |a / h| at most: the result is within
+// 1/2 + 4 u units in the last place, where a division is within 1/2.  That takes
+// reciprocal, quotient and residual inside the format's range: h and a (or a = 0)
+// between the limits here; any other pair is divided.
 template <typename T>
 struct Quot {
     T h, r;
     bool mult;
     __device__ __forceinline__ explicit Quot(T h_) : h(h_) {
-        const T big = sizeof(T) == 8 ? T(1e100) : T(1e15f);
+        const T big = sizeof(T) == 8 ? T(1e100) : T(1e15f);  // 2^332, 2^50
         mult = h > T(1) / big && h < big;
         r = mult ? Ar<T>::div(T(1), h) : T(0);
     }
+    // 2^-76 <= |a| < 2^76 (fp64: 2^-680, 2^680), or 0
+    static __device__ __forceinline__ bool inside(float a) {
+        const unsigned x = __float_as_uint(a) << 1, lo = 51u << 24, hi = 203u << 24;
+        return x - lo < hi - lo || x == 0;
+    }
+    static __device__ __forceinline__ bool inside(double a) {
+        const unsigned long long x = (unsigned long long)__double_as_longlong(a) << 1;
+        const unsigned long long lo = 343ull << 53, hi = 1703ull << 53;
+        return x - lo < hi - lo || x == 0;
+    }
     __device__ __forceinline__ T operator()(T a) const {
-        if (!mult) return Ar<T>::div(a, h);
+        if (!mult || !inside(a)) return Ar<T>::div(a, h);
         const T q = Ar<T>::mul(a, r);
         return Ar<T>::fma(Ar<T>::fma(-q, h, a), r, q);
     }

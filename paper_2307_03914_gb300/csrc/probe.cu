@@ -1,5 +1,6 @@
-// probe.cu -- measured issue rate of the SM's plain (non-tensor) fused
-// multiply-add pipes in fp32 and fp64.  These are the denominators of the ALU
+// probe.cu -- the Gram-Schmidt kernels' quotient on a caller's operands, and the
+// measured issue rate of the SM's plain (non-tensor) fused multiply-add pipes in
+// fp32 and fp64.  These are the denominators of the ALU
 // rooflines of the kernels that arithmetic, not memory, bounds: the SPAI build
 // (Householder least squares in u_f = fp32) and the Dot2 residual (fp64).  The
 // paper has no counterpart; it is a measurement aid.
@@ -9,6 +10,7 @@
 // blocks per SM.  The chains' results are folded into one store that depends
 // on all of them, so nothing is removed by the compiler.
 #include "common.cuh"
+#include "mgs.cuh"
 
 namespace bspai {
 
@@ -72,6 +74,13 @@ static int probe(int iters, cudaStream_t s, double* fma_per_s, float* ms_out) {
     return BSPAI_OK;
 }
 
+template <typename T>
+__global__ void __launch_bounds__(256) k_quotients(int n, const T* __restrict__ a, const T* __restrict__ h,
+                                                   T* __restrict__ q) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) q[i] = Quot<T>(h[i])(a[i]);
+}
+
 }  // namespace bspai
 
 using namespace bspai;
@@ -85,6 +94,20 @@ int bspai_probe_fma(bspai_prec_t prec, int32_t iters, bspai_stream_t st, double*
     if (prec == BSPAI_FP32) return probe<float>(iters, s, fma_per_s, ms);
     if (prec == BSPAI_FP64) return probe<double>(iters, s, fma_per_s, ms);
     return set_error(BSPAI_ERR_UNSUPPORTED, "bspai_probe_fma: prec must be FP32 or FP64");
+}
+
+int bspai_probe_quotients(bspai_prec_t prec, int32_t n, const void* a, const void* h, void* q, bspai_stream_t st) {
+    if (n < 0 || (n > 0 && (!a || !h || !q))) return set_error(BSPAI_ERR_INVALID, "bspai_probe_quotients: bad arguments");
+    if (prec != BSPAI_FP32 && prec != BSPAI_FP64)
+        return set_error(BSPAI_ERR_UNSUPPORTED, "bspai_probe_quotients: prec must be FP32 or FP64");
+    if (n == 0) return BSPAI_OK;
+    cudaStream_t s = (cudaStream_t)st;
+    const unsigned blocks = (unsigned)ceil_div(n, 256);
+    if (prec == BSPAI_FP32) k_quotients<float><<<blocks, 256, 0, s>>>(n, (const float*)a, (const float*)h, (float*)q);
+    else k_quotients<double><<<blocks, 256, 0, s>>>(n, (const double*)a, (const double*)h, (double*)q);
+    note_launch();
+    CUDA_LAUNCH_CHECK();
+    return BSPAI_OK;
 }
 
 }  // extern "C"
