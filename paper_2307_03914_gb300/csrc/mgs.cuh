@@ -121,7 +121,7 @@ __device__ __forceinline__ float pk_sum(float2 a) { return __fadd_rn(a.x, a.y); 
 // the residual rounded once (d3), all |d| <= u = 2^-24 or 2^-53, what is rounded last
 // differs from a / h by (2 u) (2 u) |a / h| at most: the result is within
 // 1/2 + 4 u units in the last place, where a division is within 1/2.  That takes
-// reciprocal, quotient and residual inside the format's range: h and a (or a = 0)
+// reciprocal, quotient and residual inside the format's range: h and a (or a = +0)
 // between the limits here; any other pair is divided.
 template <typename T>
 struct Quot {
@@ -132,15 +132,15 @@ struct Quot {
         mult = h > T(1) / big && h < big;
         r = mult ? Ar<T>::div(T(1), h) : T(0);
     }
-    // 2^-76 <= |a| < 2^76 (fp64: 2^-680, 2^680), or 0
+    // 2^-76 <= |a| < 2^76 (fp64: 2^-680, 2^680), or +0 (-0 would come out +0)
     static __device__ __forceinline__ bool inside(float a) {
-        const unsigned x = __float_as_uint(a) << 1, lo = 51u << 24, hi = 203u << 24;
-        return x - lo < hi - lo || x == 0;
+        const unsigned b = __float_as_uint(a), x = b << 1, lo = 51u << 24, hi = 203u << 24;
+        return x - lo < hi - lo || b == 0;
     }
     static __device__ __forceinline__ bool inside(double a) {
-        const unsigned long long x = (unsigned long long)__double_as_longlong(a) << 1;
-        const unsigned long long lo = 343ull << 53, hi = 1703ull << 53;
-        return x - lo < hi - lo || x == 0;
+        const unsigned long long b = (unsigned long long)__double_as_longlong(a);
+        const unsigned long long x = b << 1, lo = 343ull << 53, hi = 1703ull << 53;
+        return x - lo < hi - lo || b == 0;
     }
     __device__ __forceinline__ T operator()(T a) const {
         if (!mult || !inside(a)) return Ar<T>::div(a, h);

@@ -70,4 +70,6 @@ def test_divides_outside_its_range(dtype):
     odd = np.resize(np.array([np.inf, -np.inf, np.nan, f.tiny, f.tiny / 2], dtype), 200_000)
     with np.errstate(all="ignore"):
         for x, y in [(small, h), (large, h), (any_a, edge), (zeros, h), (odd, h)]:
-            assert np.array_equal(_quot(x, y), x / y, equal_nan=True)
+            q = _quot(x, y)
+            assert np.array_equal(q, x / y, equal_nan=True)
+            assert np.array_equal(np.signbit(q) | np.isnan(q), np.signbit(x / y) | np.isnan(q))
