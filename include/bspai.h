@@ -139,7 +139,9 @@ typedef struct {
     int32_t gmres_cycles[32];  /* GMRES cycles of each refinement step (1 unless capped) */
 } bspai_solve_info_t;
 
-/* Kernel-class timing, recorded with CUDA events on the launching stream. */
+/* Kernel-class timing, recorded with CUDA events on the launching stream.  A
+ * GMRES run that takes all its steps in one launch (see bspai_gmres_plan), and the
+ * GMRES launches of a batched solve, count as BSPAI_K_MGS with their products. */
 enum {
     BSPAI_K_SPAI = 0, BSPAI_K_BUCKET = 1, BSPAI_K_SPMV_A = 2, BSPAI_K_BSPMV = 3,
     BSPAI_K_MGS = 4, BSPAI_K_RESIDUAL = 5, BSPAI_K_UPDATE = 6, BSPAI_K_OTHER = 7,
@@ -387,7 +389,7 @@ int bspai_gmres(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_t u_g, b
  * applies the Givens rotations); poll_bulk = 1 when the on-chip kernel reads
  * the grid reductions' slots by bulk copies into shared memory instead of by
  * loads (at least 16 KB of each basis vector per block and at least 64
- * blocks), 0 otherwise.  Every kernel takes the basis in groups of 1 to 8
+ * blocks), 0 otherwise.  Every kernel takes the basis in groups of 2, 4 or 8
  * vectors, one reduction per group.  (A system of at most 32,768 rows that
  * max_blocks leaves room for, whose A and M have short rows, takes all its
  * steps in one launch instead, with the same Gram-Schmidt in groups of 8 on
