@@ -1,7 +1,8 @@
 // gmres.cu -- left-preconditioned MGS-GMRES and the refinement loop of Alg 3.1.
 //
-// Per Arnoldi step j (the "hot loop" of the method) three launches run on the
-// solve's stream, with no host synchronisation between steps:
+// A small system with short rows runs all its Arnoldi steps in one launch
+// (k_gmres_coop).  Otherwise, per step j (the "hot loop" of the method), three
+// launches run on the solve's stream, with no host synchronisation between steps:
 //   w = A v_j               (u_p, SELL SpMV)                       spmv.cu
 //   z = M w -> V(:, j+1)    (Alg 2.3 bucketed SpMV, stored in u_g) spmv.cu
 //   k_mgs                   (cooperative, persistent)              this file
@@ -347,7 +348,7 @@ __device__ __forceinline__ void mgs_kernel(typename I::type* __restrict__ V, int
                 unit_load<I>(R, zg, u, z + u * I::PN);
             }
         }
-        const MgsIo io{tags, hq, tri, &st->bar, tmo, G, bulk, blockIdx.x == 0, blockIdx.x == 0, nullptr};
+        const MgsIo io{tags, hq, tri, &st->bar, tmo, G, bulk, blockIdx.x == 0, blockIdx.x == 0};
         unsigned seq = seq0, phase = 0, par = 0;
         T hz;
         if (!mgs_passes<I>(sh, io, R, z, smraw, zs, V + r0, ldv, j, tag, seq, phase, par, hz)) {
@@ -448,8 +449,20 @@ __global__ void __launch_bounds__(BD, 1) k_mgs_res2(float* __restrict__ V, int64
 // A row's entries -- columns and values as the product uses them -- are kept in shared
 // memory for the run (at most kCoopRow per row of each matrix, in one fp64 bucket or
 // one or two narrow ones), so that a product waits for one load, x's, instead of a
-// chain of three.  (A launch whose matrices have longer rows stays with the products'
-// own kernels: at 17 and 24 entries per row they took 32 us a step against 57 here.)
+// chain of three.  The others that are admitted (coop_blocks) are read from memory.
+// Measured, 40 steps, us, three launches per step -> one launch per run:
+//   u_g = fp32, kept:          fp32 or fp32 + fp16, 5 to 9 entries per row, n = 1,000 to
+//                              32,000     1,258 to 1,372 -> 631 to 987; fp64 M 1,339 to 1,413 -> 930 to 1,240
+//   u_g = fp32, from memory:   mixes with fp64, 5 entries  1,344 to 1,482 -> 932 to 1,374;
+//                              fp32, 10 to 16 entries  1,281 to 1,425 -> 977 to 1,362;
+//                              fp64 M, 10 to 16 entries, n = 1,000  1,388 to 1,544 -> 1,248 to 1,433,
+//                              n = 8,192 and 32,000  1,363 to 1,509 -> 1,435 to 1,737
+//   u_g = fp64, 5 to 9:        n = 1,000  1,775 to 1,893 -> 1,726 to 1,926; 8,192  1,741 to 1,847 -> 1,793
+//                              to 1,900; 32,000  2,251 to 2,419 -> 1,951 to 2,173
+//   u_g = fp64, 10 to 16:      n = 1,000  1,880 to 1,891 -> 1,912 to 2,115; 8,192  1,834 to 1,861 -> 1,959
+//                              to 2,145; 32,000  2,331 to 2,390 -> 2,155 to 2,348
+// The line does not look at precisions; the fp64 products of 10 to 16 entries are what it
+// costs, 16 % at most.
 constexpr int kCoopBD = 512;
 constexpr int kCoopRow = 9;
 constexpr int kCoopMax = 32;  // row blocks at most (fp64: twice as many)
@@ -614,7 +627,7 @@ __global__ void __launch_bounds__(kCoopBD, 1) k_gmres_coop(const __grid_constant
     R.nb = r1 > r0 ? (int)(r1 - r0) : 0;
     const int64_t r = r0 + R.row(0);
     const int rows = R.valid(0) / (int)sizeof(T);  // of this thread
-    const MgsIo io{tags, hq, tri, &st->bar, tmo, G, 0, blockIdx.x == 0, blockIdx.x == 0, nullptr};
+    const MgsIo io{tags, hq, tri, &st->bar, tmo, G, 0, blockIdx.x == 0, blockIdx.x == 0};
     // the matrices' rows into shared memory
     CoopCache ca, cm;
     int na[VW], nm[VW];
@@ -1047,7 +1060,7 @@ static int choose_mgs(GmresWork& W) {
     const size_t es = W.ug == BSPAI_FP64 ? 8 : 4;
     const ResInstance ri = es == 8 ? pick_res<double>(chunk) : pick_res<float>(chunk);
     if (!ri.fn) return BSPAI_OK;
-        if (es == 8 && ri.per_thread > 1) {
+    if (es == 8 && ri.per_thread > 1) {
         // fp64 is bound by the narrow fp64 pipe of the SMs that hold rows: spread the rows
         // over more blocks, down to just over half of the instance's capacity (per vector
         // at n = 262,144: 9.0 us before, 3.6 with groups of 4 on 127 blocks)
@@ -1080,8 +1093,9 @@ static int choose_mgs(GmresWork& W) {
 
 // The row blocks of the whole run in one launch (k_gmres_coop), or 0: an order that few
 // enough blocks cover, with a further block left for the rotations, and matrices whose
-// rows are short (by their widest slices; packed widths are rounded up to fours, and a
-// longer row is read from memory).
+// rows are short: buckets whose widest slices add up to twice what is kept of a row, since
+// packed widths are rounded up to fours (8 for a 5- or 7-point stencil's rows, in each of
+// two buckets).  A longer row is read from memory; both sides measured above.
 static int coop_blocks(const GmresWork& W, const BMDev& A, const BMDev& M) {
     const int per = W.ug == BSPAI_FP64 ? kCoopBD : 2 * kCoopBD;
     const int64_t G = ceil_div(W.n, per);
@@ -1766,29 +1780,31 @@ int bspai_gmres_noalloc(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_
     W.sms = o.max_blocks > 0 && o.max_blocks < num_sms() ? o.max_blocks : num_sms();
     W.G = (occ >= 2 ? 2 : 1) * W.sms;
     const size_t kx = (size_t)W.kmax;
-    size_t off[12];
-    size_t sz[11] = {es * (size_t)W.ldv * (kx + 1), es * (size_t)W.ldv, es * 2 * (size_t)W.G, sizeof(GmresState),
-                     sizeof(double) * (kx + 1) * kx, sizeof(double) * (kx + 1), sizeof(double) * (kx + 1),
-                     sizeof(double) * (kx + 2), sizeof(double) * (kx + 1), sizeof(double) * 4,
-                     sizeof(unsigned long long) * 4 * kTagMaxBlocks};
+    const size_t sz[9] = {es * (size_t)W.ldv * (kx + 1), es * (size_t)W.ldv, sizeof(GmresState),
+                          sizeof(double) * (kx + 1) * kx, sizeof(double) * (kx + 1), sizeof(double) * (kx + 1),
+                          sizeof(double) * (kx + 2), sizeof(double) * (kx + 1), sizeof(double) * 4};
+    size_t off[10];
     off[0] = 0;
-    for (int i = 0; i < 11; ++i) off[i + 1] = align256(off[i] + sz[i]);
-    if (off[11] > kNoallocScratchBytes)
+    for (int i = 0; i < 9; ++i) off[i + 1] = align256(off[i] + sz[i]);
+    // partial sums and slots of one value per reduction, which had their place in the block
+    // before the reductions' own buffers (carve): still counted, so that the limit is where it was
+    const size_t need = off[9] + align256(es * 2 * (size_t)W.G) + align256(sizeof(unsigned long long) * 4 * kTagMaxBlocks);
+    if (need > kNoallocScratchBytes)
         return set_error(BSPAI_ERR_INVALID,
                          "bspai_gmres_noalloc: n = %d with kmax = %d needs %zu bytes of scratch; the fixed block "
                          "holds %zu bytes (lower kmax or use bspai_gmres)",
-                         W.n, W.kmax, off[11], kNoallocScratchBytes);
+                         W.n, W.kmax, need, kNoallocScratchBytes);
     unsigned char* base = nullptr;
     BSPAI_TRY(noalloc_scratch_address(reinterpret_cast<void**>(&base)));
     W.V = base + off[0];
     W.w = base + off[1];
-    W.st = reinterpret_cast<GmresState*>(base + off[3]);
-    W.H = reinterpret_cast<double*>(base + off[4]);
-    W.cs = reinterpret_cast<double*>(base + off[5]);
-    W.sn = reinterpret_cast<double*>(base + off[6]);
-    W.g = reinterpret_cast<double*>(base + off[7]);
-    W.y = reinterpret_cast<double*>(base + off[8]);
-    W.norms = reinterpret_cast<double*>(base + off[9]);
+    W.st = reinterpret_cast<GmresState*>(base + off[2]);
+    W.H = reinterpret_cast<double*>(base + off[3]);
+    W.cs = reinterpret_cast<double*>(base + off[4]);
+    W.sn = reinterpret_cast<double*>(base + off[5]);
+    W.g = reinterpret_cast<double*>(base + off[6]);
+    W.y = reinterpret_cast<double*>(base + off[7]);
+    W.norms = reinterpret_cast<double*>(base + off[8]);
     if (W.aux_bytes() > kNoallocAuxBytes)
         return set_error(BSPAI_ERR_INVALID, "bspai_gmres_noalloc: the reductions' buffers need %zu bytes",
                          W.aux_bytes());

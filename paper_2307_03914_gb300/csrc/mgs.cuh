@@ -244,7 +244,6 @@ struct MgsIo {
     int bulk;     // poll by bulk copies (instances that have them compiled in)
     bool tri_out; // this block writes new rows of tri
     bool hq_out;  // this block publishes the coefficients
-    double* hcol; // or (not null) writes them here: the column of H itself
 };
 
 template <typename T, int VW_, int NU_, int BD_, int GB_, int S_, bool BULK_, bool ZS_>
@@ -293,17 +292,6 @@ __device__ __forceinline__ void mgs_shared_init(MgsShared<I>& sh) {  // one thre
     }
     mbar_init_fence();
 }
-// before a further mgs_shared_init on the same storage (one thread, every copy complete)
-template <class I>
-__device__ __forceinline__ void mgs_shared_retire(MgsShared<I>& sh) {
-#pragma unroll
-    for (int s = 0; s < I::S; ++s) mbar_inval(&sh.full[s]);
-    if constexpr (I::BULK) {
-#pragma unroll
-        for (int w = 0; w < I::NPW; ++w) mbar_inval(&sh.mbar[w]);
-    }
-}
-
 template <class I>
 struct MgsRows {  // the rows of one thread of one block
     int nb;       // rows of the block
@@ -594,10 +582,7 @@ __device__ __forceinline__ bool mgs_passes(MgsShared<I>& sh, const MgsIo& io, co
         if (w == 0) {
             const T h = group_coeff<T, GB>(rowt, sh.tot, cnt, last);
             if (lane < GB) sh.h[lane] = lane < cnt ? h : T(0);
-            if (lane < cnt) {
-                if (io.hcol) io.hcol[i0 + lane] = (double)h;
-                else if (io.hq_out) tag_publish(h, io.hq + (int64_t)(i0 + lane) * TagWords<T>::W, hq_tag);
-            }
+            if (lane < cnt && io.hq_out) tag_publish(h, io.hq + (int64_t)(i0 + lane) * TagWords<T>::W, hq_tag);
         }
         __syncthreads();
         if (!*(volatile int*)&sh.ok) {
@@ -632,7 +617,7 @@ __device__ __forceinline__ bool mgs_passes(MgsShared<I>& sh, const MgsIo& io, co
         ++seq;
         mgs_arrive<I>(sh, io, seq, w == 0);
         mgs_poll<I>(sh, io, seq, w == 0, phase);
-        if (w == 0 && lane == 0 && io.hq_out && !io.hcol)
+        if (w == 0 && lane == 0 && io.hq_out)
             tag_publish(Ar<T>::sqrt(sh.tot[0]), io.hq + (int64_t)(j + 1) * TagWords<T>::W, hq_tag);
         __syncthreads();
     }
