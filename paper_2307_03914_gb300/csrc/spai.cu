@@ -48,13 +48,16 @@ int launch_row_absmax_inv(int n, const int32_t* row_ptr, const double* val, doub
 // the limits that the choice asks about (team_pays), and the candidates up to which it does
 constexpr int kNarrowRows = 32, kTallRows = 96, kWideLeast = 196, kSampleL = 256;
 
-// |I_k| of a column by a warp, from its row of M at base: the distinct columns among its
-// candidates, eight per lane (at most kSampleL; |J| <= 32).  Above `enough`, any larger number.
-__device__ __forceinline__ int shadow_rows(int64_t base, int nJ, int enough, const int32_t* __restrict__ mcol,
+// |I_k| of a column by a warp, from its row of M at base: its candidates (at most kSampleL, |J| <= 32)
+// into an open-addressing table of 2 kSampleL columns in shared memory, each counted once; above
+// `enough`, any larger number.  (Comparing the candidates with one another took 53 registers in
+// place of 32, and with them half of the warps that k_spai_sizes has in flight: a build at 128^3
+// 2,618 us against 2,590, one of 16,384 columns of 11 scattered entries 486 against 478.)
+__device__ __forceinline__ int shadow_rows(int64_t base, int nJ, int enough, int* table, const int32_t* __restrict__ mcol,
                                            const int32_t* __restrict__ arp, const int32_t* __restrict__ acol) {
     constexpr unsigned full = 0xffffffffu;
-    constexpr int E = kSampleL / 32;
     const int lane = threadIdx.x & 31;
+    for (int t = lane; t < 2 * kSampleL; t += 32) table[t] = -1;
     int rb = 0, len = 0;
     if (lane < nJ) {
         const int j = mcol[base + (int64_t)lane * kSlice];
@@ -68,39 +71,30 @@ __device__ __forceinline__ int shadow_rows(int64_t base, int nJ, int enough, con
         if (lane >= o) end += v;
     }
     const int L = __shfl_sync(full, end, 31);
-    int c[E];
-    bool fresh[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        c[e] = -1;
-        if (32 * e >= L) continue;
-        // candidate idx is entry idx - (end - len) of the row whose entries end above it
-        const int idx = lane + 32 * e;
+    const int first = rb - (end - len);  // candidate i is entry first + i of the first row that ends above i
+    __syncwarp();
+    int nI = 0;
+    for (int i0 = 0; i0 < L && nI <= enough; i0 += 32) {
+        int fresh = 0;
+        const int i = i0 + lane;
         int at = -1;
         for (int q = 0; q < nJ; ++q) {
-            const int hi = __shfl_sync(full, end, q), first = __shfl_sync(full, rb - (end - len), q);
-            if (at < 0 && idx < hi) at = first + idx;
+            const int hi = __shfl_sync(full, end, q), f = __shfl_sync(full, first, q);
+            if (at < 0 && i < hi) at = f + i;
         }
-        if (at >= 0) c[e] = acol[at];
-    }
-#pragma unroll
-    for (int e = 0; e < E; ++e) fresh[e] = c[e] >= 0;
-    int nI = 0;  // among the first 32 (e0 + 1) candidates
-#pragma unroll
-    for (int e0 = 0; e0 < E; ++e0) {
-        if (32 * e0 >= L || nI > enough) break;
-#pragma unroll 4
-        for (int l = 0; l < 32; ++l) {
-            const int v = __shfl_sync(full, c[e0], l);  // (an absent one, -1, meets none that is fresh)
-            if (lane > l && c[e0] == v) fresh[e0] = false;
-#pragma unroll
-            for (int e = e0 + 1; e < E; ++e)
-                if (c[e] == v) fresh[e] = false;
+        if (at >= 0) {
+            const int c = acol[at];
+            for (unsigned h = (unsigned)c * 2654435761u >> 23;; h = (h + 1) & (2 * kSampleL - 1)) {
+                const int old = atomicCAS(table + h, -1, c);
+                fresh = old == -1;
+                if (old == -1 || old == c) break;
+            }
         }
-        nI += __popc(__ballot_sync(full, fresh[e0]));
+        nI += __popc(__ballot_sync(full, fresh));
     }
     return nI;
 }
+static_assert(kSampleL == 256, "the table's hash takes nine bits");
 
 // Per column: |J_k| and the candidate count sum_{j in J_k} |row j of A|; their maxima go to
 // out[0], out[1].  One column per warp of every `every`-th block (0: none) is looked at further: out[2]
@@ -108,6 +102,7 @@ __device__ __forceinline__ int shadow_rows(int64_t base, int nJ, int enough, con
 __global__ void __launch_bounds__(256) k_spai_sizes(int n, const int64_t* __restrict__ msptr, const int32_t* __restrict__ mcol,
                              const int32_t* __restrict__ mrowlen, const int32_t* __restrict__ arp,
                              const int32_t* __restrict__ acol, int every, int* __restrict__ out) {
+    __shared__ int s_table[8][2 * kSampleL], s_seen[8];
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t base = k < n ? msptr[k >> 5] + (k & 31) : 0;
     int nJ = 0, L = 0;
@@ -126,9 +121,9 @@ __global__ void __launch_bounds__(256) k_spai_sizes(int n, const int64_t* __rest
         const bool in = __shfl_sync(0xffffffffu, (int)(k < n), src) != 0;
         int rows = sl;
         if (in && sl > kNarrowRows && sl <= kSampleL && sj <= 32)
-            rows = shadow_rows(sb, sj, sl < kWideLeast ? kNarrowRows : kTallRows, mcol, arp, acol);
+            rows = shadow_rows(sb, sj, sl < kWideLeast ? kNarrowRows : kTallRows, s_table[threadIdx.x >> 5], mcol,
+                               arp, acol);
         // the block's three counts in one word
-        __shared__ int s_seen[8];
         const int seen = block_combine(!in ? 0 : 1 + (rows > kNarrowRows ? 1 << 8 : 0) + (rows > kTallRows ? 1 << 16 : 0),
                                        0, s_seen, [](int a, int b) { return a + b; });
         if (threadIdx.x == 0) {
@@ -578,7 +573,8 @@ int bspai_build(const bspai_csr_t* A, const bspai_csr_t* P, double spai_eps, bsp
             note_launch();
             const int blocks = (int)ceil_div(n, 256);
             // about 2,048 columns of a large system are looked at further; none where it would cost what
-            // a team gives (5 to 8 us; at 3,600 rows a 9-point build takes 205 us in either form)
+            // a team gives (at 3,600 rows a 9-point build takes 205 us in either form, at 10,648 a
+            // 7-point one 197 by teams, look included, and 214 by warps)
             const int every = u_f != BSPAI_FP32 || n <= 8192 ? 0 : blocks <= 256 ? 1 : blocks / 256;
             k_spai_sizes<<<(unsigned)blocks, 256, 0, s>>>(n, M->sell.sptr, M->sell.col, M->rowlen, A->row_ptr, A->col,
                                                           every, sizes);
