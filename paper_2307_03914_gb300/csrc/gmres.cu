@@ -1095,8 +1095,11 @@ static int choose_mgs(GmresWork& W) {
 // enough blocks cover, with a further block left for the rotations, and matrices whose
 // rows are short: buckets whose widest slices add up to twice what is kept of a row, since
 // packed widths are rounded up to fours (8 for a 5- or 7-point stencil's rows, in each of
-// two buckets).  A longer row is read from memory; both sides measured above.
+// two buckets).  A longer row is read from memory; both sides measured above.  A run of one
+// step in fp32 does not earn back the rows' way into shared memory (n = 1,000 and 8,192:
+// 138 and 141 us in one launch, 127 and 129 in three).
 static int coop_blocks(const GmresWork& W, const BMDev& A, const BMDev& M) {
+    if (W.ug == BSPAI_FP32 && W.kmax < 2) return 0;
     const int per = W.ug == BSPAI_FP64 ? kCoopBD : 2 * kCoopBD;
     const int64_t G = ceil_div(W.n, per);
     if (G > (int64_t)kCoopMax * (2 * kCoopBD / per) || G >= W.sms) return 0;
