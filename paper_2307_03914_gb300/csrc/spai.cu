@@ -7,7 +7,8 @@
 // so column k of M' is row k of M and column j of B is row j of A times d_j.
 //
 // In u_f = fp32 a team of threads per column holds the block in registers
-// (spai_team.cuh).  The larger blocks, and u_f = fp16, take one warp per column k:
+// (spai_team.cuh) where that is the faster form (team_pays).  Otherwise, and in
+// u_f = fp16, one warp takes a column k:
 //   J_k   = pattern of row k of M (ascending)
 //   I_k   = shadow: the union of the columns of rows J_k of A, sorted (bitonic
 //           sort of the gathered candidates in shared memory, then a
