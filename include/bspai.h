@@ -392,7 +392,7 @@ int bspai_gmres(bspai_A_h A, bspai_BM_h BM, const double* r, bspai_prec_t u_g, b
  * blocks), 0 otherwise.  Every kernel takes the basis in groups of 2, 4 or 8
  * vectors, one reduction per group.  (A system of at most 32,768 rows that
  * max_blocks leaves room for, whose A and M have short rows, takes all its
- * steps in one launch instead, with the same Gram-Schmidt in groups of 8 on
+ * steps (in fp32 two or more) in one launch instead, with the same Gram-Schmidt in groups of 8 on
  * blocks of 512 threads and its own row products in every SpMV form; the
  * order alone does not tell, so the query does not.)  A query only: nothing is launched or allocated.  n < 1:
  * BSPAI_ERR_INVALID; another u_g: BSPAI_ERR_UNSUPPORTED. */

@@ -107,3 +107,17 @@ def test_one_launch_products(B, name, ug, precs, eps, tol):
     Ah, BM, S, r = _system(B, A, precs, eps)
     for k in (1, 9, 40):
         _check(B, Ah, BM, S, r, ug, k, 0, True, tol)
+
+
+def test_a_single_fp32_step_is_no_run(B):
+    """kmax = 1: in fp32 the three launches of a step, in fp64, and from two steps on, one launch."""
+    A = W.convdiff2d(25, 41)
+    for ug in ("fp32", "fp64"):
+        Ah, BM, S, r = _system(B, A, [ug])
+        d = torch.empty(r.size, dtype=torch.float64, device="cuda")
+        counts = []
+        for k in (1, 2):
+            n0 = B.launch_count()
+            B.gmres(Ah, BM, dev(r), d, ug, ug, B.opts(tau=0.0, kmax=k))
+            counts.append(B.launch_count() - n0)
+        assert counts[0] - counts[1] == (2 if ug == "fp32" else 0), (ug, counts)
